@@ -74,7 +74,8 @@ struct GraphEntry {
 bool same_params(const PassParams &a, const PassParams &b) {
     return a.lim == b.lim && a.local_iters == b.local_iters && a.larsen_n == b.larsen_n && a.omega == b.omega &&
            a.inv2h == b.inv2h && a.floor_ == b.floor_ && a.bf16 == b.bf16 && a.h2 == b.h2 && a.scheme == b.scheme &&
-           a.tiled_f32 == b.tiled_f32 && a.tiled_fh == b.tiled_fh && a.quad_f32 == b.quad_f32 && a.quad_fh == b.quad_fh;
+           a.tiled_f32 == b.tiled_f32 && a.tiled_fh == b.tiled_fh && a.quad_f32 == b.quad_f32 &&
+           a.quad_fh == b.quad_fh && a.run_f32 == b.run_f32 && a.run_fh == b.run_fh;
 }
 
 }  // namespace
@@ -592,7 +593,8 @@ void set_valid(fld_grid_s *g, Family fam) {
 // its second buffers; the state is not changed.
 // ---------------------------------------------------------------------------
 struct TuneChoice {
-    int tiled = -1;           // blocked configuration id; launched passes: -1 two, -2 four unknowns per thread
+    int tiled = -1;           // blocked configuration id; launched passes: two unknowns per thread in tiles -1 or by
+                              // running number -3, four per thread -2
     int check_every = 64;
     double us_launched = 0.0, us_best = 0.0, us_check = 0.0;   // measured per iteration / per check
 };
@@ -616,7 +618,7 @@ std::string tune_path() {
 
 std::string tune_key(const fld_grid_s *g, Family fam, const PassParams &pp) {
     char b[192];
-    snprintf(b, sizeof(b), "v2 %dx%dx%d fam%d lim%d r%d bf%d sm%d", g->nx, g->ny, g->nz, (int)fam, pp.lim,
+    snprintf(b, sizeof(b), "v3 %dx%dx%d fam%d lim%d r%d bf%d sm%d", g->nx, g->ny, g->nz, (int)fam, pp.lim,
              pp.local_iters, pp.bf16, g->nsm);
     return b;
 }
@@ -636,7 +638,7 @@ void tune_load_locked() {
         while (!key.empty() && key.back() == ' ') key.pop_back();
         TuneChoice c;
         if (sscanf(bar + 1, "%d %d %lf %lf %lf", &c.tiled, &c.check_every, &c.us_launched, &c.us_best, &c.us_check) == 5 &&
-            c.tiled >= -2 && c.tiled < kTiledConfigs && c.check_every >= 1)
+            c.tiled >= -3 && c.tiled < kTiledConfigs && c.check_every >= 1)
             g_tune[key] = c;
     }
     fclose(fp);
@@ -670,10 +672,11 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
     const int n = 16;   // iterations per timing, a multiple of every depth
     TuneChoice c;
     double best = INFINITY;
-    for (int cand = -2; cand < kTiledConfigs; ++cand) {
+    for (int cand = -3; cand < kTiledConfigs; ++cand) {
         double t = INFINITY;
         PassParams pc = pp;
         pc.quad_f32 = pc.quad_fh = cand == -2 ? 1 : 0;
+        pc.run_f32 = pc.run_fh = cand == -3 ? 1 : 0;
         for (int rep = 0; rep < 3; ++rep) {   // the first is a warm-up
             FLD_CK(cudaEventRecord(g->evb0, g->stream));
             if (cand < 0) {
@@ -722,6 +725,7 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
 fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *pp, int *ce) {
     pp->tiled_f32 = pp->tiled_fh = -1;
     pp->quad_f32 = pp->quad_fh = p->cells_per_thread == 4 ? 1 : 0;
+    pp->run_f32 = pp->run_fh = -1;
     *ce = p->check_every > 0 ? p->check_every : 64;
     if (p->scheme != FLD_SCHEME_RED_BLACK || p->precision == FLD_PREC_FP64) return FLD_OK;
     fld_status st = FLD_OK;
@@ -761,13 +765,15 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
             if ((st = ensure_tiled(g, c.tiled)) != FLD_OK) return st;
             if (c.tiled >= 0) FLD_CK(tiled_prepare(fam, c.tiled, *pp));
             const int shape = c.tiled >= 0 ? c.tiled : -1;
-            const int quad = c.tiled == -2 ? 1 : 0;
+            const int quad = c.tiled == -2 ? 1 : 0, run = c.tiled == -3 ? 1 : c.tiled == -1 ? 0 : -1;
             if (fam == FAM_F32) {
                 pp->tiled_f32 = shape;
                 pp->quad_f32 = quad;
+                pp->run_f32 = run;
             } else {
                 pp->tiled_fh = shape;
                 pp->quad_fh = quad;
+                pp->run_fh = run;
             }
         }
         if (k == 0 && p->check_every <= 0) *ce = c.check_every;

@@ -29,6 +29,9 @@ struct PassParams {
     int tiled_f32 = -1, tiled_fh = -1;
     // launched passes: four unknowns per thread (128-bit loads) instead of two
     int quad_f32 = 0, quad_fh = 0;
+    // launched pair passes: items by running number (1), in tiles (0) or by the
+    // length of a row (-1)
+    int run_f32 = -1, run_fh = -1;
 };
 
 // Device fields of one grid (padded layout unless noted).

@@ -326,6 +326,49 @@ __device__ __forceinline__ float ff_den(const FFTerms &t, float ah, float Dp) {
     return __fadd_rn(__fadd_rn(ah, 3.0f * Dp), 0.5f * t.C);
 }
 
+// n / d for n < 2^31 by one multiplication: m = ceil(2^(32+s) / d) with
+// 2^s < d <= 2^(s+1) exceeds 2^(32+s) / d by less than 2^(s+1) / d, which moves no
+// quotient of such n (Granlund and Montgomery 1994).
+struct Divisor {
+    uint32_t m = 0, s = 0;       // m = 0: d = 1
+    void set(uint32_t d) {
+        m = s = 0;
+        if (d <= 1) return;
+        while ((2u << s) < d) ++s;
+        m = (uint32_t)(((1ull << (32 + s)) + d - 1) / d);
+    }
+    __device__ __forceinline__ uint32_t quot(uint32_t n) const { return m ? __umulhi(n, m) >> s : n; }
+};
+
+// How the threads of a launched pass take the items (pairs, or single unknowns
+// for the float-float pass) of its rows: 32 x 4 tiles of a plane, or, running,
+// item e of all rows by thread e, so that rows shorter or a little longer than
+// a multiple of 32 items leave no lanes idle.
+struct PassIndex {
+    uint32_t per_row, total;     // items per row, items of all ny x nz rows
+    Divisor by_items, by_rows;
+};
+constexpr int kPassThreads = 128;
+
+template <bool RUN>
+__device__ __forceinline__ bool pass_item(const Layout &L, const PassIndex &ix, int &t, int &J, int &K) {
+    if (RUN) {
+        const uint32_t e = blockIdx.x * (uint32_t)kPassThreads + threadIdx.x;
+        if (e >= ix.total) return false;
+        const uint32_t row = ix.by_items.quot(e);
+        t = (int)(e - row * ix.per_row);
+        K = (int)ix.by_rows.quot(row);
+        J = (int)row - K * L.ny + 1;
+        ++K;
+    } else {
+        t = blockIdx.x * 32 + (threadIdx.x & 31);
+        J = blockIdx.y * (kPassThreads / 32) + (threadIdx.x >> 5) + 1;
+        K = blockIdx.z + 1;
+        if (J > L.ny) return false;
+    }
+    return true;
+}
+
 // Two adjacent unknowns t, t+1 (t even) of one colour in row (J, K) per
 // thread: in the colour-split layout they are one aligned float2 of every
 // field, their x-neighbours three consecutive elements of the other colour's
@@ -424,11 +467,14 @@ __device__ __forceinline__ void tile_f32(const Layout &L, const float *__restric
     }
 }
 
-// The launched FP32 pass.  Registers are left to hold all of a thread's
-// loads in flight (48, five CTAs per SM): measured faster than capping them
-// for occupancy (six CTAs at 40 registers: 8.0 against 7.8 us per 128^3 pass).
-template <int LIM, int ROUNDS, bool BF>
-__global__ void __launch_bounds__(256, 4) k_pass2_f32(Layout L, const float *__restrict__ sp,
+// The launched FP32 pass.  Its threads wait on memory (a CDA limiter with one
+// round, a third of the arithmetic, takes 101 of 113 us per iteration at
+// 256^3), so registers are left to hold all of a thread's loads in flight (48),
+// and 128-thread CTAs, which a finished warp keeps waiting less, hold ten of
+// them per SM: 13.7 -> 13.4 us per iteration at 128^3, 113.9 -> 108.9 at 256^3
+// against 256 threads.
+template <int LIM, int ROUNDS, bool BF, bool RUN>
+__global__ void __launch_bounds__(kPassThreads, 8) k_pass2_f32(Layout L, PassIndex ix, const float *__restrict__ sp,
                                                    const float *__restrict__ ah2, const float *__restrict__ jh2,
                                                    const uint16_t *__restrict__ spb,
                                                    const uint16_t *__restrict__ sab, float h2,
@@ -436,9 +482,10 @@ __global__ void __launch_bounds__(256, 4) k_pass2_f32(Layout L, const float *__r
                                                    int lim_rt, float larsen_n, float omega, float inv2h,
                                                    float floor_, int rounds_rt) {
     pdl_launch_dependents();
-    tile_f32<LIM, ROUNDS, BF>(L, sp, ah2, jh2, spb, sab, h2, phi, D, colour, lim_rt, larsen_n, omega,
-                                           inv2h, floor_, rounds_rt, 2 * (blockIdx.x * blockDim.x + threadIdx.x),
-                                           blockIdx.y * blockDim.y + threadIdx.y + 1, blockIdx.z + 1);
+    int t, J, K;
+    if (!pass_item<RUN>(L, ix, t, J, K)) return;
+    tile_f32<LIM, ROUNDS, BF>(L, sp, ah2, jh2, spb, sab, h2, phi, D, colour, lim_rt, larsen_n, omega, inv2h, floor_,
+                              rounds_rt, 2 * t, J, K);
 }
 
 // Middle pass (phi as a hi/lo pair, FP32-summed update, cell::cell_fh):
@@ -478,10 +525,10 @@ __device__ __forceinline__ void tile_fh(const Layout &L, const float *__restrict
     }
 }
 
-// The launched hi/lo pass (64 registers, four CTAs per SM, no spills; at
-// five CTAs per SM it spilled and ran 15 % slower at 256^3).
-template <int LIM, int ROUNDS, bool BF>
-__global__ void __launch_bounds__(256, 4) k_pass2_fh(Layout L, const float *__restrict__ sp,
+// The launched hi/lo pass (64 registers, eight CTAs per SM, no spills; with 48
+// registers it spilled and ran 25 % slower at 256^3).
+template <int LIM, int ROUNDS, bool BF, bool RUN>
+__global__ void __launch_bounds__(kPassThreads, 8) k_pass2_fh(Layout L, PassIndex ix, const float *__restrict__ sp,
                                                   const float *__restrict__ ah2, const float *__restrict__ jh2,
                                                   const uint16_t *__restrict__ spb,
                                                   const uint16_t *__restrict__ sab, float h2,
@@ -489,10 +536,10 @@ __global__ void __launch_bounds__(256, 4) k_pass2_fh(Layout L, const float *__re
                                                   float *__restrict__ D, int colour, int lim_rt, float larsen_n,
                                                   float omega, float inv2h, float floor_, int rounds_rt) {
     pdl_launch_dependents();
-    tile_fh<LIM, ROUNDS, BF>(L, sp, ah2, jh2, spb, sab, h2, phi, phlo, D, colour, lim_rt, larsen_n,
-                                          omega, inv2h, floor_, rounds_rt,
-                                          2 * (blockIdx.x * blockDim.x + threadIdx.x),
-                                          blockIdx.y * blockDim.y + threadIdx.y + 1, blockIdx.z + 1);
+    int t, J, K;
+    if (!pass_item<RUN>(L, ix, t, J, K)) return;
+    tile_fh<LIM, ROUNDS, BF>(L, sp, ah2, jh2, spb, sab, h2, phi, phlo, D, colour, lim_rt, larsen_n, omega, inv2h,
+                             floor_, rounds_rt, 2 * t, J, K);
 }
 
 // Four adjacent unknowns t .. t+3 (t a multiple of 4) of one colour in row
@@ -1185,7 +1232,19 @@ inline dim3 pass_grid(const Layout &L, dim3 blk) {
     return dim3((half + blk.x - 1) / blk.x, (L.ny + blk.y - 1) / blk.y, L.nz);
 }
 
-// two unknowns per thread (k_pass2_*): ceil(half / 2) threads per half row
+// Grid and item numbering of a launched pass with the given number of items per
+// row; run: by running number (pass_item).
+inline dim3 item_grid(const Layout &L, int per_row, bool run, PassIndex *ix) {
+    ix->per_row = (uint32_t)per_row;
+    ix->total = (uint32_t)per_row * (uint32_t)L.ny * (uint32_t)L.nz;
+    ix->by_items.set((uint32_t)per_row);
+    ix->by_rows.set((uint32_t)L.ny);
+    if (run) return dim3((ix->total + kPassThreads - 1) / kPassThreads);
+    const int rows = kPassThreads / 32;
+    return dim3((per_row + 31) / 32, (L.ny + rows - 1) / rows, L.nz);
+}
+
+// work items of the multi-grid pass: ceil(half / 2) pairs per half row
 inline dim3 pass2_grid(const Layout &L, dim3 blk) {
     const int pairs = ((L.nx + 1) / 2 + 1) / 2;
     return dim3((pairs + blk.x - 1) / blk.x, (L.ny + blk.y - 1) / blk.y, L.nz);
@@ -1195,6 +1254,18 @@ inline dim3 pass2_grid(const Layout &L, dim3 blk) {
 inline dim3 pass4_grid(const Layout &L, dim3 blk) {
     const int quads = ((L.nx + 1) / 2 + 3) / 4;
     return dim3((quads + blk.x - 1) / blk.x, (L.ny + blk.y - 1) / blk.y, L.nz);
+}
+
+// Whether a pass takes its items by running number: as asked (0 tiles, 1
+// running), or (-1) where 32-wide tiles would leave more than a sixth of the
+// lanes idle.  Measured at the ends: 33 items a row (131 x 97 x 115 hi/lo) 20.6 ->
+// 13.4 us per iteration, 40 (160^3) 51.8 -> 37.0; 32 (128^3) 17.0 tiled against
+// 17.7 running.
+// A launch's y and z extents end at 65535: longer grids run.
+inline bool pass_runs(const Layout &L, int per_row, int asked) {
+    if ((L.ny + kPassThreads / 32 - 1) / (kPassThreads / 32) > 65535 || L.nz > 65535) return true;
+    if (asked >= 0) return asked != 0;
+    return 6 * per_row < 5 * 32 * ((per_row + 31) / 32);
 }
 
 inline dim3 vox_block() { return dim3(32, 8, 1); }
@@ -1285,7 +1356,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
                         cudaStream_t s) {
     const dim3 blk(32, 8, 1);
     const dim3 grd = pass_grid(L, blk);
-    const dim3 grd2 = pass2_grid(L, blk);
+    const int pairs = ((L.nx + 1) / 2 + 1) / 2;
     switch (fam) {
     case FAM_F32:
     case FAM_FH:
@@ -1306,17 +1377,21 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
         }
         if (fam == FAM_FH) break;
         {
-        auto pick = [&](auto bf) {
-            constexpr bool B = decltype(bf)::value;
-            auto k = k_pass2_f32<-1, 0, B>;
-            if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass2_f32<LIM_LP, 2, B>;
-            else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass2_f32<LIM_KERSHAW, 2, B>;
-            else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_f32<LIM_LARSEN, 2, B>;
-            return launch_pdl(k, grd2, blk, s, L, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.D, colour,
+        auto pick = [&](auto bf, auto run) {
+            constexpr bool B = decltype(bf)::value, R = decltype(run)::value;
+            auto k = k_pass2_f32<-1, 0, B, R>;
+            if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass2_f32<LIM_LP, 2, B, R>;
+            else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass2_f32<LIM_KERSHAW, 2, B, R>;
+            else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_f32<LIM_LARSEN, 2, B, R>;
+            PassIndex ix;
+            const dim3 g2 = item_grid(L, pairs, R, &ix);
+            return launch_pdl(k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.D, colour,
                               p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_,
                               p.local_iters);
         };
-        return p.bf16 ? pick(std::true_type{}) : pick(std::false_type{});
+        if (pass_runs(L, pairs, p.run_f32))
+            return p.bf16 ? pick(std::true_type{}, std::true_type{}) : pick(std::false_type{}, std::true_type{});
+        return p.bf16 ? pick(std::true_type{}, std::false_type{}) : pick(std::false_type{}, std::false_type{});
         }
     default:
         break;
@@ -1331,17 +1406,21 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
                           (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_, p.local_iters);
     }
     case FAM_FH: {
-        auto pick = [&](auto bf) {
-            constexpr bool B = decltype(bf)::value;
-            auto k = k_pass2_fh<-1, 0, B>;
-            if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass2_fh<LIM_LP, 2, B>;
-            else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass2_fh<LIM_KERSHAW, 2, B>;
-            else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_fh<LIM_LARSEN, 2, B>;
-            return launch_pdl(k, grd2, blk, s, L, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
+        auto pick = [&](auto bf, auto run) {
+            constexpr bool B = decltype(bf)::value, R = decltype(run)::value;
+            auto k = k_pass2_fh<-1, 0, B, R>;
+            if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass2_fh<LIM_LP, 2, B, R>;
+            else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass2_fh<LIM_KERSHAW, 2, B, R>;
+            else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_fh<LIM_LARSEN, 2, B, R>;
+            PassIndex ix;
+            const dim3 g2 = item_grid(L, pairs, R, &ix);
+            return launch_pdl(k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
                               f.D, colour, p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h,
                               (float)p.floor_, p.local_iters);
         };
-        return p.bf16 ? pick(std::true_type{}) : pick(std::false_type{});
+        if (pass_runs(L, pairs, p.run_fh))
+            return p.bf16 ? pick(std::true_type{}, std::true_type{}) : pick(std::false_type{}, std::true_type{});
+        return p.bf16 ? pick(std::true_type{}, std::false_type{}) : pick(std::false_type{}, std::false_type{});
     }
     case FAM_F64:
         k_pass_d<<<grd, blk, 0, s>>>(L, f.sp64, f.ah264, f.jh264, f.phi64, f.D64, colour, p.lim, p.larsen_n,
