@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <initializer_list>
 #include <map>
 #include <tuple>
 #include <mutex>
@@ -75,7 +76,8 @@ bool same_params(const PassParams &a, const PassParams &b) {
     return a.lim == b.lim && a.local_iters == b.local_iters && a.larsen_n == b.larsen_n && a.omega == b.omega &&
            a.inv2h == b.inv2h && a.floor_ == b.floor_ && a.bf16 == b.bf16 && a.h2 == b.h2 && a.scheme == b.scheme &&
            a.tiled_f32 == b.tiled_f32 && a.tiled_fh == b.tiled_fh && a.quad_f32 == b.quad_f32 &&
-           a.quad_fh == b.quad_fh && a.run_f32 == b.run_f32 && a.run_fh == b.run_fh;
+           a.quad_fh == b.quad_fh && a.run_f32 == b.run_f32 && a.run_fh == b.run_fh &&
+           a.rows_f32 == b.rows_f32 && a.rows_fh == b.rows_fh && a.rows_ff == b.rows_ff;
 }
 
 }  // namespace
@@ -103,6 +105,11 @@ struct fld_grid_s {
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, evb0 = nullptr, evb1 = nullptr;
     long long kernels = 0;                       // kernel launches issued so far
     fld_grid_s *coarse = nullptr;                // nested solves: the next 2x coarser grid (owned)
+    // device memory that the fields above and below are parts of (alloc_block):
+    // the fields, inputs and reduction scratch; FP64 fields; snapshots; second
+    // buffers of the sweeps; Anderson history
+    void *block = nullptr, *block_f64 = nullptr, *block_snap = nullptr, *block_snap64 = nullptr, *block_alt = nullptr,
+         *block_and = nullptr;
     // last good state of a solve (float family: phi, lo, D; FP64: phi, D)
     float *snap_phi = nullptr, *snap_lo = nullptr, *snap_D = nullptr;
     double *snap_phi64 = nullptr, *snap_D64 = nullptr;
@@ -110,6 +117,7 @@ struct fld_grid_s {
     AndersonBuffers anderson{};
     int anderson_slots = 0;
     int nsm = 0;
+    RowsTile rtile[3] = {{0, 0}, {0, 0}, {0, 0}};   // tiles of whole-iteration launches (rows_slot)
     // temporally blocked sweeps: the other buffers of the ping-pong pair, the
     // kernels' timeout flag and the TMA descriptors (made on first use)
     float *alt_phi = nullptr, *alt_D = nullptr, *alt_lo = nullptr;
@@ -125,20 +133,41 @@ struct fld_grid_s {
 
 namespace {
 
+// Several device buffers from one cudaMalloc (a call costs about 28 us, and a
+// first solve made more than a dozen): each part starts on 512 bytes; *base owns
+// them all.  Nothing is allocated on failure.
+struct Part {
+    void **p;
+    size_t bytes;
+};
+bool alloc_block(void **base, std::initializer_list<Part> parts, size_t *total = nullptr) {
+    size_t n = 0;
+    for (const Part &q : parts) n += (q.bytes + 511) & ~(size_t)511;
+    if (cudaMalloc(base, n) != cudaSuccess) {
+        (void)cudaGetLastError();
+        *base = nullptr;
+        return false;
+    }
+    char *at = (char *)*base;
+    for (const Part &q : parts) {
+        *q.p = at;
+        at += (q.bytes + 511) & ~(size_t)511;
+    }
+    if (total) *total = n;
+    return true;
+}
+
 long long nvox(const fld_grid_s *g) { return (long long)g->nx * g->ny * g->nz; }
 
 fld_status ensure_f64(fld_grid_s *g) {
     if (g->f.phi64) return FLD_OK;
     const size_t bytes = sizeof(double) * (size_t)g->L.total;
-    double **ptrs[6] = {&g->f.sp64, &g->f.ah264, &g->f.jh264, &g->f.phi64, &g->f.D64, &g->f.Df64};
-    for (double **p : ptrs) {
-        cudaError_t e = cudaMalloc((void **)p, bytes);
-        if (e != cudaSuccess) {
-            (void)cudaGetLastError();
-            return fail(FLD_ERR_OOM, "cudaMalloc of the FP64 fields failed");
-        }
-        FLD_CK(cudaMemsetAsync(*p, 0, bytes, g->stream));
-    }
+    size_t n = 0;
+    if (!alloc_block(&g->block_f64,
+                     {{(void **)&g->f.sp64, bytes}, {(void **)&g->f.ah264, bytes}, {(void **)&g->f.jh264, bytes},
+                      {(void **)&g->f.phi64, bytes}, {(void **)&g->f.D64, bytes}, {(void **)&g->f.Df64, bytes}}, &n))
+        return fail(FLD_ERR_OOM, "cudaMalloc of the FP64 fields failed");
+    FLD_CK(cudaMemsetAsync(g->block_f64, 0, n, g->stream));
     return FLD_OK;
 }
 
@@ -172,9 +201,8 @@ fld_status ensure_jacobi(fld_grid_s *g, Family fam) {
 }
 
 void free_anderson(fld_grid_s *g) {
-    void *ptrs[] = {g->anderson.g, g->anderson.f, g->anderson.x, g->anderson.part, g->anderson.dots};
-    for (void *q : ptrs)
-        if (q) cudaFree(q);
+    if (g->block_and) cudaFree(g->block_and);
+    g->block_and = nullptr;
     g->anderson = AndersonBuffers{};
     g->anderson_slots = 0;
 }
@@ -190,12 +218,11 @@ fld_status ensure_anderson(fld_grid_s *g, int m) {
     }
     const size_t n = (size_t)g->L.total;
     AndersonBuffers &b = g->anderson;
-    if (cudaMalloc((void **)&b.g, sizeof(float2) * n * m) != cudaSuccess ||
-        cudaMalloc((void **)&b.f, sizeof(float) * n * m) != cudaSuccess ||
-        cudaMalloc((void **)&b.x, sizeof(float2) * n) != cudaSuccess ||
-        cudaMalloc((void **)&b.part, sizeof(double) * kAndersonMax * 4 * (size_t)g->nsm) != cudaSuccess ||
-        cudaMalloc((void **)&b.dots, sizeof(double) * kAndersonMax) != cudaSuccess) {
-        (void)cudaGetLastError();
+    if (!alloc_block(&g->block_and, {{(void **)&b.g, sizeof(float2) * n * m},
+                                     {(void **)&b.f, sizeof(float) * n * m},
+                                     {(void **)&b.x, sizeof(float2) * n},
+                                     {(void **)&b.part, sizeof(double) * kAndersonMax * 4 * (size_t)g->nsm},
+                                     {(void **)&b.dots, sizeof(double) * kAndersonMax}})) {
         free_anderson(g);
         return fail(FLD_ERR_OOM, "cudaMalloc of the Anderson history failed");
     }
@@ -322,19 +349,43 @@ fld_status read_result(fld_grid_s *g, double out[2]) {
     return FLD_OK;
 }
 
+// The other buffers of the ping-pong pair, and the blocked kernels' status.
+fld_status ensure_alt(fld_grid_s *g) {
+    if (g->alt_phi) return FLD_OK;
+    const size_t nb = sizeof(float) * (size_t)g->L.total;
+    if (!alloc_block(&g->block_alt, {{(void **)&g->alt_phi, nb}, {(void **)&g->alt_D, nb}, {(void **)&g->alt_lo, nb},
+                                     {(void **)&g->tiled_status, sizeof(int)}}))
+        return fail(FLD_ERR_OOM, "cudaMalloc of the sweeps' second buffers failed");
+    FLD_CK(cudaMemsetAsync(g->tiled_status, 0, sizeof(int), g->stream));
+    return FLD_OK;
+}
+
+// Whole iterations per launch pay where the launch and one memory latency are
+// most of a colour pass (measured, us per iteration against two launched passes:
+// 24^3 2.6 / 4.3, 32^3 2.7 / 4.2, hi/lo 3.3 / 4.2; 40^3 hi/lo 5.0 / 6.8; 50^3 5.3 /
+// 5.5; 64^3 8.5 / 6.1): above this size they are not tried.
+constexpr long long kRowsMaxVoxels = 250000;
+int rows_slot(Family fam) { return fam == FAM_F32 ? 0 : fam == FAM_FH ? 1 : 2; }
+
+// Tile of the whole-iteration launches of family fam; *ok: the grid can run them.
+fld_status ensure_rows(fld_grid_s *g, Family fam, const PassParams &pp, bool *ok) {
+    *ok = false;
+    if (nvox(g) > kRowsMaxVoxels) return FLD_OK;
+    RowsTile &t = g->rtile[rows_slot(fam)];
+    if (t.TJ == 0) t = rows_tile(g->L, fam, g->nsm);
+    if (t.TJ == 0) return FLD_OK;
+    fld_status st = ensure_alt(g);
+    if (st != FLD_OK) return st;
+    FLD_CK(rows_prepare(fam, pp));
+    *ok = true;
+    return FLD_OK;
+}
+
 // Buffers and TMA descriptors of blocked configuration `id`.
 fld_status ensure_tiled(fld_grid_s *g, int id) {
     if (id < 0) return FLD_OK;
-    if (!g->alt_phi) {
-        const size_t nb = sizeof(float) * (size_t)g->L.total;
-        if (cudaMalloc((void **)&g->alt_phi, nb) != cudaSuccess || cudaMalloc((void **)&g->alt_D, nb) != cudaSuccess ||
-            cudaMalloc((void **)&g->alt_lo, nb) != cudaSuccess ||
-            cudaMalloc((void **)&g->tiled_status, sizeof(int)) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return fail(FLD_ERR_OOM, "cudaMalloc of the blocked sweeps' buffers failed");
-        }
-        FLD_CK(cudaMemsetAsync(g->tiled_status, 0, sizeof(int), g->stream));
-    }
+    fld_status st = ensure_alt(g);
+    if (st != FLD_OK) return st;
     if (!g->maps_ok[id]) {
         FLD_CK(tiled_maps(g->L, id, g->f.phi, g->f.D, g->f.phlo, &g->maps[id][0]));
         FLD_CK(tiled_maps(g->L, id, g->alt_phi, g->alt_D, g->alt_lo, &g->maps[id][1]));
@@ -510,6 +561,16 @@ fld_status enqueue_iterations(fld_grid_s *g, Family fam, const PassParams &pp, i
             g->tiled_used = true;
         }
     }
+    if (fam == FAM_F32 ? pp.rows_f32 : fam == FAM_FH ? pp.rows_fh : fam == FAM_FF ? pp.rows_ff : 0) {
+        // whole iterations per launch, an even number of them (ping-pong); the
+        // first also brings the ghosts to the second buffers
+        if (!g->alt_phi) return fail(FLD_ERR_STATE, "whole-iteration sweeps were not prepared");
+        float *const a[3] = {g->f.phi, g->f.D, g->f.phlo}, *const b[3] = {g->alt_phi, g->alt_D, g->alt_lo};
+        for (; done < (iters & ~1); ++done)
+            FLD_CK(launch_rows(fam, g->L, g->f, pp, g->rtile[rows_slot(fam)], done & 1 ? b : a, done & 1 ? a : b,
+                               done == 0, g->stream));
+        if (nk) *nk = done + 2LL * (iters - done);
+    }
     for (int it = done; it < iters; ++it)
         for (int colour = 0; colour < 2; ++colour) FLD_CK(launch_pass(fam, g->L, g->f, pp, colour, g->stream));
     return FLD_OK;
@@ -594,7 +655,7 @@ void set_valid(fld_grid_s *g, Family fam) {
 // ---------------------------------------------------------------------------
 struct TuneChoice {
     int tiled = -1;           // blocked configuration id; launched passes: two unknowns per thread in tiles -1 or by
-                              // running number -3, four per thread -2
+                              // running number -3, four per thread -2; whole iterations -4
     int check_every = 64;
     double us_launched = 0.0, us_best = 0.0, us_check = 0.0;   // measured per iteration / per check
 };
@@ -638,7 +699,7 @@ void tune_load_locked() {
         while (!key.empty() && key.back() == ' ') key.pop_back();
         TuneChoice c;
         if (sscanf(bar + 1, "%d %d %lf %lf %lf", &c.tiled, &c.check_every, &c.us_launched, &c.us_best, &c.us_check) == 5 &&
-            c.tiled >= -3 && c.tiled < kTiledConfigs && c.check_every >= 1)
+            c.tiled >= -4 && c.tiled < kTiledConfigs && c.check_every >= 1)
             g_tune[key] = c;
     }
     fclose(fp);
@@ -656,11 +717,15 @@ void tune_store_locked(const std::string &key, const TuneChoice &c) {
 
 // Time the candidates of family fam on g (state in the family's fields).
 fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParams &pp, Family fam, TuneChoice *out) {
-    for (int id = 0; id < kTiledConfigs; ++id) {
+    const int ncfg = fam == FAM_FF ? 0 : kTiledConfigs;   // the float-float family has no blocked form
+    for (int id = 0; id < ncfg; ++id) {
         fld_status st = ensure_tiled(g, id);
         if (st != FLD_OK) return st;
         FLD_CK(tiled_prepare(fam, id, pp));
     }
+    bool rows = false;
+    if (fld_status st = ensure_rows(g, fam, pp, &rows); st != FLD_OK) return st;
+    if (fld_status st = ensure_alt(g); st != FLD_OK) return st;
     const size_t nb = sizeof(float) * (size_t)g->L.total;
     FLD_CK(cudaMemcpyAsync(g->alt_phi, g->f.phi, nb, cudaMemcpyDeviceToDevice, g->stream));
     FLD_CK(cudaMemcpyAsync(g->alt_D, g->f.D, nb, cudaMemcpyDeviceToDevice, g->stream));
@@ -672,14 +737,21 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
     const int n = 16;   // iterations per timing, a multiple of every depth
     TuneChoice c;
     double best = INFINITY;
-    for (int cand = -3; cand < kTiledConfigs; ++cand) {
+    for (int cand = -4; cand < ncfg; ++cand) {
+        if (cand == -4 && !rows) continue;
+        if (fam == FAM_FF && (cand == -2 || cand == -3)) continue;   // one launched form
         double t = INFINITY;
         PassParams pc = pp;
         pc.quad_f32 = pc.quad_fh = cand == -2 ? 1 : 0;
         pc.run_f32 = pc.run_fh = cand == -3 ? 1 : 0;
         for (int rep = 0; rep < 3; ++rep) {   // the first is a warm-up
             FLD_CK(cudaEventRecord(g->evb0, g->stream));
-            if (cand < 0) {
+            if (cand == -4) {
+                const float *const a[3] = {g->f.phi, g->f.D, g->f.phlo};
+                float *const b[3] = {g->alt_phi, g->alt_D, g->alt_lo};
+                for (int it = 0; it < n; ++it)
+                    FLD_CK(launch_rows(fam, g->L, g->f, pc, g->rtile[rows_slot(fam)], a, b, it == 0, g->stream));
+            } else if (cand < 0) {
                 for (int it = 0; it < n; ++it)
                     for (int colour = 0; colour < 2; ++colour) FLD_CK(launch_pass(fam, g->L, fa, pc, colour, g->stream));
             } else {
@@ -699,7 +771,7 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
             c.tiled = cand;
         }
     }
-    g->tiled_used = true;   // surface a timeout of the timed blocked launches at the next check
+    if (ncfg > 0) g->tiled_used = true;   // surface a timeout of the timed blocked launches at the next check
     c.us_best = best;
     // one residual check, as the solve takes it (kernels + 16-byte readback)
     double tc = INFINITY;
@@ -726,6 +798,7 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
     pp->tiled_f32 = pp->tiled_fh = -1;
     pp->quad_f32 = pp->quad_fh = p->cells_per_thread == 4 ? 1 : 0;
     pp->run_f32 = pp->run_fh = -1;
+    pp->rows_f32 = pp->rows_fh = pp->rows_ff = 0;
     *ce = p->check_every > 0 ? p->check_every : 64;
     if (p->scheme != FLD_SCHEME_RED_BLACK || p->precision == FLD_PREC_FP64) return FLD_OK;
     fld_status st = FLD_OK;
@@ -738,8 +811,10 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
         pp->tiled_f32 = pp->tiled_fh = id;
     }
     if (p->temporal_depth != 0 && p->check_every > 0) return FLD_OK;
-    const Family fams[2] = {p->precision == FLD_PREC_PAIR ? FAM_FH : FAM_F32, FAM_FH};
-    const int nfam = p->precision == FLD_PREC_MIXED ? 2 : 1;
+    const Family fams[3] = {p->precision == FLD_PREC_PAIR ? FAM_FH : FAM_F32, FAM_FH, FAM_FF};
+    // (the float-float family has a choice on small grids only)
+    const bool small = p->temporal_depth == 0 && nvox(g) <= kRowsMaxVoxels;
+    const int nfam = p->precision != FLD_PREC_MIXED ? 1 : small ? 3 : 2;
     for (int k = 0; k < nfam; ++k) {
         const Family fam = fams[k];
         const std::string key = tune_key(g, fam, *pp);
@@ -764,13 +839,18 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
         if (p->temporal_depth == 0) {
             if ((st = ensure_tiled(g, c.tiled)) != FLD_OK) return st;
             if (c.tiled >= 0) FLD_CK(tiled_prepare(fam, c.tiled, *pp));
+            if (c.tiled == -4) {
+                bool ok = false;
+                if ((st = ensure_rows(g, fam, *pp, &ok)) != FLD_OK) return st;
+                (fam == FAM_F32 ? pp->rows_f32 : fam == FAM_FH ? pp->rows_fh : pp->rows_ff) = ok ? 1 : 0;
+            }
             const int shape = c.tiled >= 0 ? c.tiled : -1;
             const int quad = c.tiled == -2 ? 1 : 0, run = c.tiled == -3 ? 1 : c.tiled == -1 ? 0 : -1;
             if (fam == FAM_F32) {
                 pp->tiled_f32 = shape;
                 pp->quad_f32 = quad;
                 pp->run_f32 = run;
-            } else {
+            } else if (fam == FAM_FH) {
                 pp->tiled_fh = shape;
                 pp->quad_fh = quad;
                 pp->run_fh = run;
@@ -835,27 +915,27 @@ fld_status validate_inputs(fld_grid_s *g, const float *st, const float *alb, con
     return FLD_OK;
 }
 
+// The safeguard's snapshot of the family's state.
+bool ensure_snapshot(fld_grid_s *g, Family fam) {
+    const size_t nf = sizeof(float) * (size_t)g->L.total, nd = sizeof(double) * (size_t)g->L.total;
+    if (fam == FAM_F64)
+        return g->snap_phi64 || alloc_block(&g->block_snap64, {{(void **)&g->snap_phi64, nd}, {(void **)&g->snap_D64, nd}});
+    return g->snap_phi || alloc_block(&g->block_snap, {{(void **)&g->snap_phi, nf}, {(void **)&g->snap_lo, nf},
+                                                      {(void **)&g->snap_D, nf}});
+}
+
 // Everything a solve may allocate on the device, allocated before it starts
 // (so admission by free memory sees it, and no allocation falls inside the
 // solve): the safeguard's snapshot of the single-precision state, and, for a
 // MIXED solve with the FP64 stop test, the FP64 fields and their snapshot.
 fld_status preallocate(fld_grid_s *g, const fld_solve_params *p) {
-    const size_t nf = sizeof(float) * (size_t)g->L.total, nd = sizeof(double) * (size_t)g->L.total;
     const bool f64 = p->precision == FLD_PREC_FP64 || (p->precision == FLD_PREC_MIXED && p->fp64_verify);
     if (f64) {
         fld_status st = ensure_f64(g);
         if (st != FLD_OK) return st;
     }
-    bool ok = true;
-    if (!g->snap_phi)
-        ok = cudaMalloc((void **)&g->snap_phi, nf) == cudaSuccess && cudaMalloc((void **)&g->snap_lo, nf) == cudaSuccess &&
-             cudaMalloc((void **)&g->snap_D, nf) == cudaSuccess;
-    if (ok && f64 && !g->snap_phi64)
-        ok = cudaMalloc((void **)&g->snap_phi64, nd) == cudaSuccess && cudaMalloc((void **)&g->snap_D64, nd) == cudaSuccess;
-    if (!ok) {
-        (void)cudaGetLastError();
+    if (!ensure_snapshot(g, FAM_F32) || (f64 && !ensure_snapshot(g, FAM_F64)))
         return fail(FLD_ERR_OOM, "cudaMalloc of the solve's buffers failed");
-    }
     return FLD_OK;
 }
 
@@ -863,25 +943,12 @@ fld_status preallocate(fld_grid_s *g, const fld_solve_params *p) {
 fld_status snapshot(fld_grid_s *g, Family fam, bool save) {
     const size_t nf = sizeof(float) * (size_t)g->L.total, nd = sizeof(double) * (size_t)g->L.total;
     if (fam == FAM_F64) {
-        if (!g->snap_phi64) {
-            if (cudaMalloc((void **)&g->snap_phi64, nd) != cudaSuccess ||
-                cudaMalloc((void **)&g->snap_D64, nd) != cudaSuccess) {
-                (void)cudaGetLastError();
-                return fail(FLD_ERR_OOM, "cudaMalloc of the solve snapshot failed");
-            }
-        }
+        if (!ensure_snapshot(g, fam)) return fail(FLD_ERR_OOM, "cudaMalloc of the solve snapshot failed");
         double *a[2] = {g->f.phi64, g->f.D64}, *b[2] = {g->snap_phi64, g->snap_D64};
         for (int i = 0; i < 2; ++i)
             FLD_CK(cudaMemcpyAsync(save ? b[i] : a[i], save ? a[i] : b[i], nd, cudaMemcpyDeviceToDevice, g->stream));
     } else {
-        if (!g->snap_phi) {
-            if (cudaMalloc((void **)&g->snap_phi, nf) != cudaSuccess ||
-                cudaMalloc((void **)&g->snap_lo, nf) != cudaSuccess ||
-                cudaMalloc((void **)&g->snap_D, nf) != cudaSuccess) {
-                (void)cudaGetLastError();
-                return fail(FLD_ERR_OOM, "cudaMalloc of the solve snapshot failed");
-            }
-        }
+        if (!ensure_snapshot(g, fam)) return fail(FLD_ERR_OOM, "cudaMalloc of the solve snapshot failed");
         float *a[3] = {g->f.phi, g->f.phlo, g->f.D}, *b[3] = {g->snap_phi, g->snap_lo, g->snap_D};
         for (int i = 0; i < 3; ++i)
             FLD_CK(cudaMemcpyAsync(save ? b[i] : a[i], save ? a[i] : b[i], nf, cudaMemcpyDeviceToDevice, g->stream));
@@ -1132,26 +1199,34 @@ fld_status fld_create_grid(int nx, int ny, int nz, double h, void *stream, fld_g
     }
     const size_t fb = sizeof(float) * (size_t)g->L.total;
     const size_t ub = sizeof(float) * (size_t)nvox(g);
-    float **pf[7] = {&g->f.sp, &g->f.ah2, &g->f.jh2, &g->f.phi, &g->f.phlo, &g->f.D, &g->f.Df};
-    float **pu[3] = {&g->f.sigma_t, &g->f.albedo, &g->f.jsrc};
-    fld_status st = FLD_OK;
-    for (float **p : pf)
-        if (st == FLD_OK && cudaMalloc((void **)p, fb) != cudaSuccess) st = FLD_ERR_OOM;
-    for (float **p : pu)
-        if (st == FLD_OK && cudaMalloc((void **)p, ub) != cudaSuccess) st = FLD_ERR_OOM;
     g->f.partial_cap = reduction_blocks(g->L);
-    if (st == FLD_OK && cudaMalloc((void **)&g->f.partials, sizeof(double) * 2 * (size_t)g->f.partial_cap) != cudaSuccess)
+    // grids small enough for whole-iteration launches get their second buffers
+    // here; the scratch D of the checks, free during the sweeps, is one of them
+    const size_t alt = nvox(g) <= kRowsMaxVoxels ? fb : 0;
+    float *second[2] = {nullptr, nullptr};
+    int *status = nullptr;
+    size_t bytes = 0;
+    fld_status st = FLD_OK;
+    if (!alloc_block(&g->block,
+                     {{(void **)&g->f.sp, fb}, {(void **)&g->f.ah2, fb}, {(void **)&g->f.jh2, fb},
+                      {(void **)&g->f.phi, fb}, {(void **)&g->f.phlo, fb}, {(void **)&g->f.D, fb},
+                      {(void **)&g->f.Df, fb}, {(void **)&g->f.sigma_t, ub}, {(void **)&g->f.albedo, ub},
+                      {(void **)&g->f.jsrc, ub}, {(void **)&second[0], alt}, {(void **)&second[1], alt},
+                      {(void **)&status, sizeof(int)},
+                      {(void **)&g->f.result, sizeof(double) * 2},
+                      {(void **)&g->f.partials, sizeof(double) * 2 * (size_t)g->f.partial_cap}}, &bytes))
         st = FLD_ERR_OOM;
-    if (st == FLD_OK && cudaMalloc((void **)&g->f.result, sizeof(double) * 2) != cudaSuccess) st = FLD_ERR_OOM;
+    if (st == FLD_OK && alt) {
+        g->alt_phi = second[0];
+        g->alt_D = g->f.Df;
+        g->alt_lo = second[1];
+        g->tiled_status = status;
+    }
     if (st == FLD_OK && (cudaEventCreate(&g->ev0) != cudaSuccess || cudaEventCreate(&g->ev1) != cudaSuccess ||
                          cudaEventCreate(&g->evb0) != cudaSuccess || cudaEventCreate(&g->evb1) != cudaSuccess))
         st = FLD_ERR_CUDA;
-    if (st == FLD_OK) {
-        for (float **p : pf)
-            if (cudaMemsetAsync(*p, 0, fb, g->stream) != cudaSuccess) st = FLD_ERR_CUDA;
-        for (float **p : pu)
-            if (cudaMemsetAsync(*p, 0, ub, g->stream) != cudaSuccess) st = FLD_ERR_CUDA;
-    }
+    if (st == FLD_OK && cudaMemsetAsync(g->block, 0, (size_t)((char *)g->f.result - (char *)g->block), g->stream) != cudaSuccess)
+        st = FLD_ERR_CUDA;
     if (st != FLD_OK) {
         (void)cudaGetLastError();
         fld_destroy(g);
@@ -1172,19 +1247,14 @@ void fld_destroy(fld_grid g) {
     if (g->stream) cudaStreamSynchronize(g->stream);
     for (GraphEntry &e : g->graphs)
         if (e.exec) cudaGraphExecDestroy(e.exec);
-    void *ptrs[] = {g->f.sp, g->f.ah2, g->f.jh2, g->f.phi, g->f.phlo, g->f.D, g->f.Df, g->f.sp64, g->f.ah264,
-                    g->f.jh264, g->f.phi64, g->f.D64, g->f.Df64, g->f.sigma_t, g->f.albedo, g->f.jsrc,
-                    g->f.partials, g->f.result, g->f.spb, g->f.sab, g->f.phi2, g->f.phi642, g->f.render_vol};
+    void *ptrs[] = {g->block, g->block_f64, g->block_snap, g->block_snap64, g->block_alt, g->f.spb, g->f.sab, g->f.phi2,
+                    g->f.phi642, g->f.render_vol, g->stage_rad, g->stage_cod};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (g->ev0) cudaEventDestroy(g->ev0);
     if (g->ev1) cudaEventDestroy(g->ev1);
     if (g->evb0) cudaEventDestroy(g->evb0);
     if (g->evb1) cudaEventDestroy(g->evb1);
-    void *snaps[] = {g->snap_phi, g->snap_lo, g->snap_D, g->snap_phi64, g->snap_D64, g->alt_phi, g->alt_D,
-                     g->alt_lo, g->tiled_status, g->stage_rad, g->stage_cod};
-    for (void *p : snaps)
-        if (p) cudaFree(p);
     free_anderson(g);
     if (g->own_stream && g->stream) cudaStreamDestroy(g->stream);
     delete g;

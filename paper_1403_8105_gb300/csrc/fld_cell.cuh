@@ -51,9 +51,23 @@ __device__ __forceinline__ float limiter_fast(int kind, float larsen_n, float R)
     }
 }
 
+// limiter_fast without branches for Levermore-Pomraning: both forms, then a
+// select (the same bits).  For kernels with few warps per SM, whose threads
+// update several unknowns: without branches between them their chains of
+// dependent operations overlap.
+__device__ __forceinline__ float limiter_fast_sel(int kind, float larsen_n, float R) {
+    if (kind != LIM_LP) return limiter_fast(kind, larsen_n, R);
+    const float S = lp_series_f(R);
+    const float r = fast_rcp(R);
+    const float e = 2.0f * fast_rcp(__fsub_rn(__expf(2.0f * R), 1.0f));
+    const float tail = R < 9.0f ? e : 0.0f;
+    const float G = r * __fadd_rn(__fsub_rn(1.0f, r), tail);
+    return R < 1.0f ? S : G;
+}
+
 // Arithmetic of one FP32 point update from its gathered values: the
 // neighbours' phi and D, its own phi and medium; returns the new phi and D.
-template <int LIM, int ROUNDS>
+template <int LIM, int ROUNDS, bool SEL = false>
 __device__ __forceinline__ void cell_f32(float p0, const float ps[6], const float Ds[6], float s_, float ah, float jj,
                                          int lim_rt, float larsen_n, float omega, float inv2h, float floor_,
                                          int rounds_rt, float &phi_new, float &D_new) {
@@ -79,7 +93,7 @@ __device__ __forceinline__ void cell_f32(float p0, const float ps[6], const floa
     for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : 64); ++r) {
         if (ROUNDS == 0 && r >= local_iters) break;
         const float R = gmax * fast_rcp(fmaxf(s_ * __fadd_rn(p0, delta), floor_));     // Eq. 35
-        Dp = limiter_fast(lim, larsen_n, R) * inv_sp;                          // Eq. 33
+        Dp = (SEL ? limiter_fast_sel(lim, larsen_n, R) : limiter_fast(lim, larsen_n, R)) * inv_sp;                          // Eq. 33
         delta = fmaf(0.5f * Dp, A, base) * fast_rcp(fmaf(3.0f, Dp, den0));   // Eq. 32
     }
     phi_new = fmaf(omega, delta, p0);                                          // Eq. 36
@@ -90,7 +104,7 @@ __device__ __forceinline__ void cell_f32(float p0, const float ps[6], const floa
 // summed in plain FP32 with the approximate D of the bulk sweeps -- about the
 // cost of the FP32 pass, reaching residuals a few times above the
 // float-float pass's.  cell_fh is the arithmetic of one point.
-template <int LIM, int ROUNDS>
+template <int LIM, int ROUNDS, bool SEL = false>
 __device__ __forceinline__ void cell_fh(float p0, float p0lo, const float ps[6], const float ls[6],
                                         const float Ds[6], float s_, float ah, float jj, int lim_rt, float larsen_n,
                                         float omega, float inv2h, float floor_, int rounds_rt, float &hi_new,
@@ -119,8 +133,83 @@ __device__ __forceinline__ void cell_fh(float p0, float p0lo, const float ps[6],
     for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : 64); ++r) {
         if (ROUNDS == 0 && r >= local_iters) break;
         const float R = gmax * fast_rcp(fmaxf(s_ * __fadd_rn(p0, delta), floor_));
-        Dp = limiter_fast(lim, larsen_n, R) * inv_sp;
+        Dp = (SEL ? limiter_fast_sel(lim, larsen_n, R) : limiter_fast(lim, larsen_n, R)) * inv_sp;
         delta = fmaf(0.5f * Dp, A, base) * fast_rcp(fmaf(3.0f, Dp, den0));
+    }
+    const ff nw = ff_add_f(ff{p0, p0lo}, __fmul_rn(omega, delta));
+    hi_new = nw.hi;
+    lo_new = nw.lo;
+    D_new = Dp;
+}
+
+// Terms of the residual-form update that do not depend on D_p, shared by the
+// sweep and the residual kernel so both evaluate the same discrete equation
+// bit for bit:  A = sum_s d_s,  B = sum_s D_s d_s,  C = sum_s D_s,
+// base = jh2 - ah2 phi_p + B/2, and the central differences.  A and B are
+// compensated sums (Ogita-Rump-Oishi style): each difference d_s =
+// phi_s - phi_p is formed exactly as a pair (TwoSum of the high words plus
+// the low words), each product D_s d_s exactly by TwoProd, and the running
+// sums carry their rounding errors in a separate low word.
+struct FFTerms {
+    ff A, base;
+    float C, gx, gy, gz;
+};
+
+__device__ __forceinline__ FFTerms ff_terms(float p0, float p0lo, const float ps[6], const float ls[6],
+                                            const float Ds[6], float ah, float jj) {
+    FFTerms t;
+    t.gx = __fadd_rn(__fsub_rn(ps[1], ps[0]), __fsub_rn(ls[1], ls[0]));
+    t.gy = __fadd_rn(__fsub_rn(ps[3], ps[2]), __fsub_rn(ls[3], ls[2]));
+    t.gz = __fadd_rn(__fsub_rn(ps[5], ps[4]), __fsub_rn(ls[5], ls[4]));
+    float Ah = 0.0f, Al = 0.0f, Bh = 0.0f, Bl = 0.0f, C = 0.0f;
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+        const ff dh = two_sum(ps[s], -p0);                                  // exact high part
+        const float dl = __fadd_rn(__fsub_rn(ls[s], p0lo), dh.lo);          // low part
+        const ff a = two_sum(Ah, dh.hi);
+        Ah = a.hi;
+        Al = __fadd_rn(Al, __fadd_rn(dl, a.lo));
+        const ff pr = two_prod(Ds[s], dh.hi);
+        const float pe = fmaf(Ds[s], dl, pr.lo);
+        const ff b = two_sum(Bh, pr.hi);
+        Bh = b.hi;
+        Bl = __fadd_rn(Bl, __fadd_rn(pe, b.lo));
+        C = __fadd_rn(C, Ds[s]);
+    }
+    const ff B = fast_two_sum(Bh, Bl);
+    ff base = ff_add_f(ff_mul_f(ff{p0, p0lo}, -ah), jj);
+    t.base = ff_add(base, ff{0.5f * B.hi, 0.5f * B.lo});
+    t.A = fast_two_sum(Ah, Al);
+    t.C = C;
+    return t;
+}
+
+// S(D_p) = base + (D_p / 2) A  and  den(D_p) = ah2 + 3 D_p + C / 2.
+__device__ __forceinline__ ff ff_S(const FFTerms &t, float Dp) { return ff_add(t.base, ff_mul_f(t.A, 0.5f * Dp)); }
+__device__ __forceinline__ float ff_den(const FFTerms &t, float ah, float Dp) {
+    return __fadd_rn(__fadd_rn(ah, 3.0f * Dp), 0.5f * t.C);
+}
+
+// One point of the float-float correction pass: phi kept as a hi/lo pair, S
+// summed so the update is accurate to the pair's precision; correctly rounded
+// D (the same function the residual kernel evaluates).
+template <int LIM, int ROUNDS>
+__device__ __forceinline__ void cell_ff(float p0, float p0lo, const float ps[6], const float ls[6],
+                                        const float Ds[6], float s_, float ah, float jj, int lim_rt, float larsen_n,
+                                        float omega, float inv2h, float floor_, int rounds_rt, float &hi_new,
+                                        float &lo_new, float &D_new) {
+    const int lim = LIM >= 0 ? LIM : lim_rt;
+    const int local_iters = ROUNDS > 0 ? ROUNDS : rounds_rt;
+    const FFTerms T = ff_terms(p0, p0lo, ps, ls, Ds, ah, jj);
+    const float gmax = grad_floor_f(T.gx, T.gy, T.gz, inv2h, floor_);
+    float delta = 0.0f, Dp = 0.0f;
+#pragma unroll
+    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : 64); ++r) {
+        if (ROUNDS == 0 && r >= local_iters) break;
+        Dp = D_of_f(gmax, s_, __fadd_rn(p0, delta), floor_, lim, larsen_n);
+        const ff S = ff_S(T, Dp);
+        // delta is a correction: its rounding does not move the fixed point
+        delta = __fdividef(__fadd_rn(S.hi, S.lo), ff_den(T, ah, Dp));
     }
     const ff nw = ff_add_f(ff{p0, p0lo}, __fmul_rn(omega, delta));
     hi_new = nw.hi;

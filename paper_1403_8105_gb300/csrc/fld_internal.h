@@ -32,6 +32,8 @@ struct PassParams {
     // launched pair passes: items by running number (1), in tiles (0) or by the
     // length of a row (-1)
     int run_f32 = -1, run_fh = -1;
+    // whole iterations per launch (fld_rows.cu)
+    int rows_f32 = 0, rows_fh = 0, rows_ff = 0;
 };
 
 // Device fields of one grid (padded layout unless noted).
@@ -245,6 +247,19 @@ cudaError_t tiled_maps(const Layout &L, int id, float *phi, float *D, float *lo,
 cudaError_t launch_tiled(Family fam, int id, const Layout &L, const Fields &f, const PassParams &p,
                          const TiledMaps &src, float *dphi, float *dD, float *dlo, int *status, int nsm,
                          cudaStream_t s);
+
+// Whole iterations of small grids, one launch each (fld_rows.cu): the tile of
+// rows a CTA owns (TJ = 0: the grid's rows do not fit), the kernel's
+// shared-memory attribute (call outside stream capture), and one iteration of
+// the FP32, hi/lo or float-float family from the buffers src (phi, D, phi lo)
+// into dst; with ghosts it also copies the ghost layer.
+struct RowsTile {
+    int TJ, TK;
+};
+RowsTile rows_tile(const Layout &L, Family fam, int nsm);
+cudaError_t rows_prepare(Family fam, const PassParams &p);
+cudaError_t launch_rows(Family fam, const Layout &L, const Fields &f, const PassParams &p, const RowsTile &t,
+                        const float *const src[3], float *const dst[3], bool ghosts, cudaStream_t s);
 
 // Relative residual Rbar / jbar of Eq. 37 from the device sums r2 = sum of
 // (R_p h^2)^2 over the unknowns at least `margin` voxels from the faces and

@@ -278,68 +278,6 @@ __device__ __forceinline__ bool pass_cell(const Layout &L, int c, int t, int J, 
     return true;
 }
 
-// Terms of the residual-form update that do not depend on D_p, shared by the
-// sweep and the residual kernel so both evaluate the same discrete equation
-// bit for bit:  A = sum_s d_s,  B = sum_s D_s d_s,  C = sum_s D_s,
-// base = jh2 - ah2 phi_p + B/2, and the central differences.  A and B are
-// compensated sums (Ogita-Rump-Oishi style): each difference d_s =
-// phi_s - phi_p is formed exactly as a pair (TwoSum of the high words plus
-// the low words), each product D_s d_s exactly by TwoProd, and the running
-// sums carry their rounding errors in a separate low word.
-struct FFTerms {
-    ff A, base;
-    float C, gx, gy, gz;
-};
-
-__device__ __forceinline__ FFTerms ff_terms(float p0, float p0lo, const float ps[6], const float ls[6],
-                                            const float Ds[6], float ah, float jj) {
-    FFTerms t;
-    t.gx = __fadd_rn(__fsub_rn(ps[1], ps[0]), __fsub_rn(ls[1], ls[0]));
-    t.gy = __fadd_rn(__fsub_rn(ps[3], ps[2]), __fsub_rn(ls[3], ls[2]));
-    t.gz = __fadd_rn(__fsub_rn(ps[5], ps[4]), __fsub_rn(ls[5], ls[4]));
-    float Ah = 0.0f, Al = 0.0f, Bh = 0.0f, Bl = 0.0f, C = 0.0f;
-#pragma unroll
-    for (int s = 0; s < 6; ++s) {
-        const ff dh = two_sum(ps[s], -p0);                                  // exact high part
-        const float dl = __fadd_rn(__fsub_rn(ls[s], p0lo), dh.lo);          // low part
-        const ff a = two_sum(Ah, dh.hi);
-        Ah = a.hi;
-        Al = __fadd_rn(Al, __fadd_rn(dl, a.lo));
-        const ff pr = two_prod(Ds[s], dh.hi);
-        const float pe = fmaf(Ds[s], dl, pr.lo);
-        const ff b = two_sum(Bh, pr.hi);
-        Bh = b.hi;
-        Bl = __fadd_rn(Bl, __fadd_rn(pe, b.lo));
-        C = __fadd_rn(C, Ds[s]);
-    }
-    const ff B = fast_two_sum(Bh, Bl);
-    ff base = ff_add_f(ff_mul_f(ff{p0, p0lo}, -ah), jj);
-    t.base = ff_add(base, ff{0.5f * B.hi, 0.5f * B.lo});
-    t.A = fast_two_sum(Ah, Al);
-    t.C = C;
-    return t;
-}
-
-// S(D_p) = base + (D_p / 2) A  and  den(D_p) = ah2 + 3 D_p + C / 2.
-__device__ __forceinline__ ff ff_S(const FFTerms &t, float Dp) { return ff_add(t.base, ff_mul_f(t.A, 0.5f * Dp)); }
-__device__ __forceinline__ float ff_den(const FFTerms &t, float ah, float Dp) {
-    return __fadd_rn(__fadd_rn(ah, 3.0f * Dp), 0.5f * t.C);
-}
-
-// n / d for n < 2^31 by one multiplication: m = ceil(2^(32+s) / d) with
-// 2^s < d <= 2^(s+1) exceeds 2^(32+s) / d by less than 2^(s+1) / d, which moves no
-// quotient of such n (Granlund and Montgomery 1994).
-struct Divisor {
-    uint32_t m = 0, s = 0;       // m = 0: d = 1
-    void set(uint32_t d) {
-        m = s = 0;
-        if (d <= 1) return;
-        while ((2u << s) < d) ++s;
-        m = (uint32_t)(((1ull << (32 + s)) + d - 1) / d);
-    }
-    __device__ __forceinline__ uint32_t quot(uint32_t n) const { return m ? __umulhi(n, m) >> s : n; }
-};
-
 // How the threads of a launched pass take the items (pairs, or single unknowns
 // for the float-float pass) of its rows: 32 x 4 tiles of a plane, or, running,
 // item e of all rows by thread e, so that rows shorter or a little longer than
@@ -753,8 +691,6 @@ __device__ __forceinline__ void pass_ff_body(const Layout &L, const float *__res
                                              float *__restrict__ D, int colour, int t, int J, int K, int lim_rt,
                                              float larsen_n, float omega, float inv2h, float floor_,
                                              int rounds_rt) {
-    const int lim = LIM >= 0 ? LIM : lim_rt;
-    const int local_iters = ROUNDS > 0 ? ROUNDS : rounds_rt;
     Nbrs o;
     if (J > L.ny || !pass_cell(L, colour, t, J, K, o)) return;
     const float s_ = sp[o.own], ah = ah2[o.own], jj = jh2[o.own];
@@ -767,20 +703,11 @@ __device__ __forceinline__ void pass_ff_body(const Layout &L, const float *__res
         ls[s] = phlo[o.nb[s]];
         Ds[s] = D[o.nb[s]];
     }
-    const FFTerms T = ff_terms(p0, p0lo, ps, ls, Ds, ah, jj);
-    const float gmax = grad_floor_f(T.gx, T.gy, T.gz, inv2h, floor_);
-    float delta = 0.0f, Dp = 0.0f;
-#pragma unroll
-    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : 64); ++r) {
-        if (ROUNDS == 0 && r >= local_iters) break;
-        Dp = D_of_f(gmax, s_, __fadd_rn(p0, delta), floor_, lim, larsen_n);
-        const ff S = ff_S(T, Dp);
-        // delta is a correction: its rounding does not move the fixed point
-        delta = __fdividef(__fadd_rn(S.hi, S.lo), ff_den(T, ah, Dp));
-    }
-    const ff nw = ff_add_f(ff{p0, p0lo}, __fmul_rn(omega, delta));
-    phi[o.own] = nw.hi;
-    phlo[o.own] = nw.lo;
+    float hi, lo, Dp;
+    cell_ff<LIM, ROUNDS>(p0, p0lo, ps, ls, Ds, s_, ah, jj, lim_rt, larsen_n, omega, inv2h, floor_, rounds_rt, hi, lo,
+                         Dp);
+    phi[o.own] = hi;
+    phlo[o.own] = lo;
     D[o.own] = Dp;
 }
 

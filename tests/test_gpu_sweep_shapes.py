@@ -36,3 +36,50 @@ def test_launched_passes_by_row_length(nx, precision, bf16):
     want = state_after(shape, precision, 1, 4, bf16=bf16)
     got = state_after(shape, precision, -1, 4, bf16=bf16)
     assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+
+
+# Whole iterations per launch (small grids), chosen through a tuning cache that
+# names them: single rows and planes, rows whose first or last unknown is of
+# either colour, tiles cut at the far faces, an odd iteration left to the passes
+ROWS_SHAPES = [(1, 1, 1), (1, 1, 9), (9, 1, 6), (1, 40, 3), (2, 3, 2), (7, 9, 8), (17, 33, 31), (24, 24, 24),
+               (32, 32, 32), (40, 37, 33), (5, 6, 250)]
+FAMILIES = {"fp32": 0, "pair": 3, "mixed": 1}
+_CHILD = """
+import sys, numpy as np
+sys.path[:0] = [{root!r}, {tests!r}]
+import test_gpu_sweep_shapes as t
+out = {{}}
+for shape in t.ROWS_SHAPES:
+    for precision in t.FAMILIES:
+        for limiter, bf16 in (("lp", 0), ("larsen", 1)):
+            if precision == "mixed" and bf16:
+                bf16 = 0
+            for depth in (0, -1):
+                phi, D = t.state_after(shape, precision, depth, 5, limiter, bf16)
+                out["%s %s %s %d phi" % (shape, precision, limiter, depth)] = phi
+                out["%s %s %s %d D" % (shape, precision, limiter, depth)] = D
+np.savez({path!r}, **out)
+"""
+
+
+def test_whole_iteration_launches_equal_the_passes(tmp_path):
+    import os
+    import subprocess
+    import sys
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lines = ["v3 %dx%dx%d fam%d lim%d r2 bf%d sm%d | -4 64 0 0 0" % (s[2], s[1], s[0], fam, lim, bf, sms)
+             for s in ROWS_SHAPES for fam in (0, 1, 3) for lim in (fld.LIMITERS["lp"], fld.LIMITERS["larsen"])
+             for bf in (0, 1)]
+    cache = tmp_path / "tune.txt"
+    cache.write_text("\n".join(lines) + "\n")
+    path = str(tmp_path / "states.npz")
+    tests = os.path.dirname(os.path.abspath(__file__))
+    code = _CHILD.format(root=os.path.dirname(tests), tests=tests, path=path)
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=600,
+                   env=dict(os.environ, FLD_TUNE_CACHE=str(cache)))
+    assert len(cache.read_text().splitlines()) == len(lines)      # nothing was tuned: every form above was the one run
+    got = np.load(path)
+    for key in got.files:
+        if " 0 " in key:
+            assert np.array_equal(got[key], got[key.replace(" 0 ", " -1 ")]), key
