@@ -77,7 +77,7 @@ bool same_params(const PassParams &a, const PassParams &b) {
            a.inv2h == b.inv2h && a.floor_ == b.floor_ && a.bf16 == b.bf16 && a.h2 == b.h2 && a.scheme == b.scheme &&
            a.tiled_f32 == b.tiled_f32 && a.tiled_fh == b.tiled_fh && a.quad_f32 == b.quad_f32 &&
            a.quad_fh == b.quad_fh && a.run_f32 == b.run_f32 && a.run_fh == b.run_fh &&
-           a.rows_f32 == b.rows_f32 && a.rows_fh == b.rows_fh && a.rows_ff == b.rows_ff;
+           a.rows_f32 == b.rows_f32 && a.rows_fh == b.rows_fh && a.rows_ff == b.rows_ff && a.ff_form == b.ff_form;
 }
 
 }  // namespace
@@ -655,7 +655,8 @@ void set_valid(fld_grid_s *g, Family fam) {
 // ---------------------------------------------------------------------------
 struct TuneChoice {
     int tiled = -1;           // blocked configuration id; launched passes: two unknowns per thread in tiles -1 or by
-                              // running number -3, four per thread -2; whole iterations -4
+                              // running number -3, four per thread -2 (float-float: two with seven -1 or five
+                              // -3 CTAs per SM, one -2); whole iterations -4
     int check_every = 64;
     double us_launched = 0.0, us_best = 0.0, us_check = 0.0;   // measured per iteration / per check
 };
@@ -739,11 +740,11 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
     double best = INFINITY;
     for (int cand = -4; cand < ncfg; ++cand) {
         if (cand == -4 && !rows) continue;
-        if (fam == FAM_FF && (cand == -2 || cand == -3)) continue;   // one launched form
         double t = INFINITY;
         PassParams pc = pp;
         pc.quad_f32 = pc.quad_fh = cand == -2 ? 1 : 0;
         pc.run_f32 = pc.run_fh = cand == -3 ? 1 : 0;
+        pc.ff_form = cand == -2 ? 2 : cand == -3 ? 1 : 0;
         for (int rep = 0; rep < 3; ++rep) {   // the first is a warm-up
             FLD_CK(cudaEventRecord(g->evb0, g->stream));
             if (cand == -4) {
@@ -799,6 +800,7 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
     pp->quad_f32 = pp->quad_fh = p->cells_per_thread == 4 ? 1 : 0;
     pp->run_f32 = pp->run_fh = -1;
     pp->rows_f32 = pp->rows_fh = pp->rows_ff = 0;
+    pp->ff_form = -1;
     *ce = p->check_every > 0 ? p->check_every : 64;
     if (p->scheme != FLD_SCHEME_RED_BLACK || p->precision == FLD_PREC_FP64) return FLD_OK;
     fld_status st = FLD_OK;
@@ -812,9 +814,7 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
     }
     if (p->temporal_depth != 0 && p->check_every > 0) return FLD_OK;
     const Family fams[3] = {p->precision == FLD_PREC_PAIR ? FAM_FH : FAM_F32, FAM_FH, FAM_FF};
-    // (the float-float family has a choice on small grids only)
-    const bool small = p->temporal_depth == 0 && nvox(g) <= kRowsMaxVoxels;
-    const int nfam = p->precision != FLD_PREC_MIXED ? 1 : small ? 3 : 2;
+    const int nfam = p->precision != FLD_PREC_MIXED ? 1 : p->temporal_depth == 0 ? 3 : 2;
     for (int k = 0; k < nfam; ++k) {
         const Family fam = fams[k];
         const std::string key = tune_key(g, fam, *pp);
@@ -854,6 +854,8 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
                 pp->tiled_fh = shape;
                 pp->quad_fh = quad;
                 pp->run_fh = run;
+            } else {
+                pp->ff_form = c.tiled == -2 ? 2 : c.tiled == -3 ? 1 : c.tiled == -1 ? 0 : -1;
             }
         }
         if (k == 0 && p->check_every <= 0) *ce = c.check_every;

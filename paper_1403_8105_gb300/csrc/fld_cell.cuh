@@ -89,9 +89,8 @@ __device__ __forceinline__ void cell_f32(float p0, const float ps[6], const floa
     const float base = fmaf(0.5f, B, fmaf(-ah, p0, jj));
     const float den0 = fmaf(0.5f, C, ah);
     float delta = 0.0f, Dp = 0.0f;
-#pragma unroll
-    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : 64); ++r) {
-        if (ROUNDS == 0 && r >= local_iters) break;
+#pragma unroll(ROUNDS > 0 ? ROUNDS : 1)
+    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : local_iters); ++r) {
         const float R = gmax * fast_rcp(fmaxf(s_ * __fadd_rn(p0, delta), floor_));     // Eq. 35
         Dp = (SEL ? limiter_fast_sel(lim, larsen_n, R) : limiter_fast(lim, larsen_n, R)) * inv_sp;                          // Eq. 33
         delta = fmaf(0.5f * Dp, A, base) * fast_rcp(fmaf(3.0f, Dp, den0));   // Eq. 32
@@ -129,9 +128,8 @@ __device__ __forceinline__ void cell_fh(float p0, float p0lo, const float ps[6],
     const float base = fmaf(0.5f, B, fmaf(-ah, p0, fmaf(-ah, p0lo, jj)));
     const float den0 = fmaf(0.5f, C, ah);
     float delta = 0.0f, Dp = 0.0f;
-#pragma unroll
-    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : 64); ++r) {
-        if (ROUNDS == 0 && r >= local_iters) break;
+#pragma unroll(ROUNDS > 0 ? ROUNDS : 1)
+    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : local_iters); ++r) {
         const float R = gmax * fast_rcp(fmaxf(s_ * __fadd_rn(p0, delta), floor_));
         Dp = (SEL ? limiter_fast_sel(lim, larsen_n, R) : limiter_fast(lim, larsen_n, R)) * inv_sp;
         delta = fmaf(0.5f * Dp, A, base) * fast_rcp(fmaf(3.0f, Dp, den0));
@@ -166,11 +164,17 @@ __device__ __forceinline__ FFTerms ff_terms(float p0, float p0lo, const float ps
     for (int s = 0; s < 6; ++s) {
         const ff dh = two_sum(ps[s], -p0);                                  // exact high part
         const float dl = __fadd_rn(__fsub_rn(ls[s], p0lo), dh.lo);          // low part
+        const ff pr = two_prod(Ds[s], dh.hi);
+        const float pe = fmaf(Ds[s], dl, pr.lo);
+        if (s == 0) {                          // the sums so far are zero
+            Ah = dh.hi; Al = dl;
+            Bh = pr.hi; Bl = pe;
+            C = Ds[0];
+            continue;
+        }
         const ff a = two_sum(Ah, dh.hi);
         Ah = a.hi;
         Al = __fadd_rn(Al, __fadd_rn(dl, a.lo));
-        const ff pr = two_prod(Ds[s], dh.hi);
-        const float pe = fmaf(Ds[s], dl, pr.lo);
         const ff b = two_sum(Bh, pr.hi);
         Bh = b.hi;
         Bl = __fadd_rn(Bl, __fadd_rn(pe, b.lo));
@@ -201,17 +205,144 @@ __device__ __forceinline__ void cell_ff(float p0, float p0lo, const float ps[6],
     const int lim = LIM >= 0 ? LIM : lim_rt;
     const int local_iters = ROUNDS > 0 ? ROUNDS : rounds_rt;
     const FFTerms T = ff_terms(p0, p0lo, ps, ls, Ds, ah, jj);
-    const float gmax = grad_floor_f(T.gx, T.gy, T.gz, inv2h, floor_);
+    const DPoint pt = D_point(grad_floor_f(T.gx, T.gy, T.gz, inv2h, floor_), s_);
     float delta = 0.0f, Dp = 0.0f;
-#pragma unroll
-    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : 64); ++r) {
-        if (ROUNDS == 0 && r >= local_iters) break;
-        Dp = D_of_f(gmax, s_, __fadd_rn(p0, delta), floor_, lim, larsen_n);
+#pragma unroll(ROUNDS > 0 ? ROUNDS : 1)
+    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : local_iters); ++r) {
+        Dp = D_of_f(pt, __fadd_rn(p0, delta), floor_, lim, larsen_n);
         const ff S = ff_S(T, Dp);
         // delta is a correction: its rounding does not move the fixed point
         delta = __fdividef(__fadd_rn(S.hi, S.lo), ff_den(T, ah, Dp));
     }
     const ff nw = ff_add_f(ff{p0, p0lo}, __fmul_rn(omega, delta));
+    hi_new = nw.hi;
+    lo_new = nw.lo;
+    D_new = Dp;
+}
+
+// ---------------------------------------------------------------------------
+// cell_ff of two unknowns, one in each half of packed FP32 instructions (add /
+// fma .f32x2).  The correction pass is bound by issue: 592 instructions per
+// update, 390 of them on the FMA pipe.  A packed instruction keeps that pipe
+// busy as long as the two it replaces (measured 63 against 126 per clock and
+// SM) but takes one issue slot.  Each half rounds like the scalar instruction
+// and every sum keeps its operands and order, so both unknowns get cell_ff's bits.
+//
+// Two rules keep it so.  The assembler contracts a packed product followed by a packed
+// sum into an FMA even with explicit rounding, so products are FMAs with +0
+// (mul2), which it leaves alone.  And a difference is an FMA with -1 (sub2): the
+// product is exact.  Negated quantities (n...) save the sign changes.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long pack2(float2 a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+    float2 a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(v));
+    return a;
+}
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return fma2(a, b, both(0.0f)); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, both(-1.0f), a); }
+
+struct ff2 {
+    float2 hi, lo;
+};
+__device__ __forceinline__ ff2 two_sum2(float2 a, float2 b) {
+    const float2 s = add2(a, b);
+    const float2 bb = sub2(s, a);
+    return {s, add2(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+__device__ __forceinline__ ff2 fast_two_sum2(float2 a, float2 b) {
+    const float2 s = add2(a, b);
+    return {s, sub2(b, sub2(s, a))};
+}
+
+template <int LIM, int ROUNDS>
+__device__ __forceinline__ void cell_ff_pair(float2 p0, float2 p0lo, const float2 ps[6], const float2 ls[6],
+                                             const float2 Ds[6], float2 s_, float2 ah, float2 jj, int lim_rt,
+                                             float larsen_n, float omega, float inv2h, float floor_, int rounds_rt,
+                                             float2 &hi_new, float2 &lo_new, float2 &D_new) {
+    const int lim = LIM >= 0 ? LIM : lim_rt;
+    const int local_iters = ROUNDS > 0 ? ROUNDS : rounds_rt;
+    const float2 half = both(0.5f);
+    // the gradient (grad_floor_f)
+    const float2 gx = mul2(add2(sub2(ps[1], ps[0]), sub2(ls[1], ls[0])), both(inv2h));
+    const float2 gy = mul2(add2(sub2(ps[3], ps[2]), sub2(ls[3], ls[2])), both(inv2h));
+    const float2 gz = mul2(add2(sub2(ps[5], ps[4]), sub2(ls[5], ls[4])), both(inv2h));
+    const float2 g2 = fma2(gx, gx, fma2(gy, gy, mul2(gz, gz)));
+    const DPoint ptx = D_point(fmaxf(sqrtf(g2.x), floor_), s_.x), pty = D_point(fmaxf(sqrtf(g2.y), floor_), s_.y);
+    // ff_terms: A = sum d_s, B = sum D_s d_s (its low word negated), C = sum D_s
+    const float2 np0 = neg2(p0);
+    float2 Ah, Al, Bh, nBl, C;
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+        const ff2 dh = two_sum2(ps[s], np0);
+        const float2 dl = add2(sub2(ls[s], p0lo), dh.lo);
+        const float2 nD = neg2(Ds[s]);
+        const float2 p = mul2(Ds[s], dh.hi);
+        const float2 npe = fma2(nD, dl, fma2(nD, dh.hi, p));
+        if (s == 0) {
+            Ah = dh.hi; Al = dl;
+            Bh = p; nBl = npe;
+            C = Ds[0];
+            continue;
+        }
+        const ff2 a = two_sum2(Ah, dh.hi);
+        Ah = a.hi;
+        Al = add2(Al, add2(dl, a.lo));
+        const ff2 b = two_sum2(Bh, p);
+        Bh = b.hi;
+        nBl = add2(nBl, sub2(npe, b.lo));
+        C = add2(C, Ds[s]);
+    }
+    const float2 B = sub2(Bh, nBl);
+    const float2 nBlo = add2(nBl, sub2(B, Bh));
+    // base = j h^2 - sigma_a' h^2 phi + B / 2
+    ff2 base;
+    {
+        const float2 P = mul2(p0, ah);
+        const float2 e = fma2(neg2(p0lo), ah, fma2(np0, ah, P));
+        const float2 mh = sub2(e, P);
+        const float2 ml = sub2(e, add2(mh, P));
+        const ff2 t = two_sum2(mh, jj);
+        const ff2 u = fast_two_sum2(t.hi, add2(t.lo, ml));
+        const ff2 v = two_sum2(u.hi, mul2(B, half));
+        base = fast_two_sum2(v.hi, add2(v.lo, sub2(u.lo, mul2(nBlo, half))));
+    }
+    const ff2 A = fast_two_sum2(Ah, Al);
+    const float2 nA = neg2(A.hi), nAlo = neg2(A.lo), hC = mul2(C, half);
+    float2 delta = both(0.0f), Dp = both(0.0f);
+#pragma unroll(ROUNDS > 0 ? ROUNDS : 1)
+    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : local_iters); ++r) {
+        Dp.x = D_of_f(ptx, __fadd_rn(p0.x, delta.x), floor_, lim, larsen_n);
+        Dp.y = D_of_f(pty, __fadd_rn(p0.y, delta.y), floor_, lim, larsen_n);
+        const float2 hd = mul2(Dp, half);
+        const float2 p = mul2(A.hi, hd);
+        const float2 ne = fma2(nAlo, hd, fma2(nA, hd, p));
+        const float2 m = sub2(p, ne);
+        const float2 nml = add2(ne, sub2(m, p));
+        const ff2 t = two_sum2(base.hi, m);
+        const ff2 S = fast_two_sum2(t.hi, add2(t.lo, sub2(base.lo, nml)));
+        const float2 num = add2(S.hi, S.lo);
+        const float2 den = add2(add2(ah, mul2(Dp, both(3.0f))), hC);
+        delta = make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));
+    }
+    const ff2 t = two_sum2(p0, mul2(both(omega), delta));
+    const ff2 nw = fast_two_sum2(t.hi, add2(t.lo, p0lo));
     hi_new = nw.hi;
     lo_new = nw.lo;
     D_new = Dp;

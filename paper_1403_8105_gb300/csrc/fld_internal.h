@@ -32,6 +32,9 @@ struct PassParams {
     // launched pair passes: items by running number (1), in tiles (0) or by the
     // length of a row (-1)
     int run_f32 = -1, run_fh = -1;
+    // launched float-float passes: two unknowns per thread with seven (0) or five
+    // (1) CTAs per SM, one unknown (2), or two by the size of the grid (-1)
+    int ff_form = -1;
     // whole iterations per launch (fld_rows.cu)
     int rows_f32 = 0, rows_fh = 0, rows_ff = 0;
 };

@@ -287,6 +287,7 @@ struct PassIndex {
     Divisor by_items, by_rows;
 };
 constexpr int kPassThreads = 128;
+constexpr long long kSmallCtas = 760;      // all resident at five per SM
 
 template <bool RUN>
 __device__ __forceinline__ bool pass_item(const Layout &L, const PassIndex &ix, int &t, int &J, int &K) {
@@ -681,9 +682,58 @@ auto multi_kernel(int lim, int local_iters) {
     return k_pass2_multi<-1, 0, BF, HL>;
 }
 
-// Float-float correction pass: phi kept as a hi/lo pair, S summed so the
-// update is accurate to the pair's precision; correctly rounded D (the same
-// function the residual kernel evaluates).
+// Float-float correction pass (cell::cell_ff), two unknowns per thread in
+// packed arithmetic (cell::cell_ff_pair).
+__device__ __forceinline__ void gather_packed(const float *f, const Pair &q, float2 v[6]) {
+    const float2 xv = ld2(f, q.xv);
+    const float xe = q.left ? f[q.xv - 1] : f[q.xv + 2];
+    v[0] = q.left ? make_float2(xe, xv.x) : xv;
+    v[1] = q.left ? xv : make_float2(xv.y, xe);
+    v[2] = ld2(f, q.ym);
+    v[3] = ld2(f, q.yp);
+    v[4] = ld2(f, q.zm);
+    v[5] = ld2(f, q.zp);
+}
+
+// Registers: with seven CTAs per SM (70 registers) the passes of grids that fill
+// the GPU are fastest (us per iteration at 256^3 with 4, 6, 7, 8 CTAs: 295, 267,
+// 241, 244; one unknown per thread 268, before quotient_rn 287; at 128^3 31.3,
+// 35.0 and 36.6); left alone (90) those of small ones, whose CTAs are all
+// resident at once and only wait longer for loads taken in turns (40^3: 6.5 against 11.1).
+template <int LIM, int ROUNDS, bool RUN, int MINB>
+__global__ void __launch_bounds__(kPassThreads, MINB) k_pass2_ff(Layout L, PassIndex ix, const float *__restrict__ sp,
+                                                  const float *__restrict__ ah2, const float *__restrict__ jh2,
+                                                  float *__restrict__ phi, float *__restrict__ phlo,
+                                                  float *__restrict__ D, int colour, int lim_rt, float larsen_n,
+                                                  float omega, float inv2h, float floor_, int rounds_rt) {
+    pdl_launch_dependents();
+    int t, J, K;
+    if (!pass_item<RUN>(L, ix, t, J, K)) return;
+    Pair q;
+    pair_cells(L, colour, 2 * t, J, K, q);
+    if (!q.first) return;
+    const float2 s2 = ld2(sp, q.own), a2 = ld2(ah2, q.own), j2 = ld2(jh2, q.own);
+    pdl_wait();
+    float2 ps[6], ls[6], Ds[6], hi, lo, dn;
+    gather_packed(phi, q, ps);
+    gather_packed(phlo, q, ls);
+    gather_packed(D, q, Ds);
+    cell_ff_pair<LIM, ROUNDS>(ld2(phi, q.own), ld2(phlo, q.own), ps, ls, Ds, s2, a2, j2, lim_rt, larsen_n, omega,
+                              inv2h, floor_, rounds_rt, hi, lo, dn);
+    if (q.second) {
+        *reinterpret_cast<float2 *>(phi + q.own) = hi;
+        *reinterpret_cast<float2 *>(phlo + q.own) = lo;
+        *reinterpret_cast<float2 *>(D + q.own) = dn;
+    } else {
+        phi[q.own] = hi.x;         // the element after the last unknown is a ghost: left untouched
+        phlo[q.own] = lo.x;
+        D[q.own] = dn.x;
+    }
+}
+
+// The same pass with one unknown per thread: still the fastest on some grids of
+// about 50^3, which have too few pairs for the GPU (us per iteration at 50^3:
+// 9.2 against 10.7).
 template <int LIM, int ROUNDS>
 __device__ __forceinline__ void pass_ff_body(const Layout &L, const float *__restrict__ sp,
                                              const float *__restrict__ ah2, const float *__restrict__ jh2,
@@ -1325,12 +1375,29 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
     }
     switch (fam) {
     case FAM_FF: {
-        auto k = k_pass_ff<-1, 0>;
-        if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass_ff<LIM_LP, 2>;
-        else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass_ff<LIM_KERSHAW, 2>;
-        else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass_ff<LIM_LARSEN, 2>;
-        return launch_pdl(k, grd, blk, s, L, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour, p.lim,
-                          (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_, p.local_iters);
+        PassIndex ix;
+        if (p.ff_form == 2) {
+            auto k = k_pass_ff<-1, 0>;
+            if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass_ff<LIM_LP, 2>;
+            else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass_ff<LIM_KERSHAW, 2>;
+            else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass_ff<LIM_LARSEN, 2>;
+            return launch_pdl(k, grd, blk, s, L, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour, p.lim,
+                              (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_, p.local_iters);
+        }
+        auto pick = [&](auto run) {
+            constexpr bool R = decltype(run)::value;
+            const dim3 g2 = item_grid(L, pairs, R, &ix);
+            auto k = k_pass2_ff<-1, 0, R, 7>;
+            if (p.local_iters == 2 && p.lim == LIM_LP)
+                k = p.ff_form == 1 || (p.ff_form < 0 && (long long)g2.x * g2.y * g2.z <= kSmallCtas)
+                        ? k_pass2_ff<LIM_LP, 2, R, 5> : k_pass2_ff<LIM_LP, 2, R, 7>;
+            else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass2_ff<LIM_KERSHAW, 2, R, 7>;
+            else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_ff<LIM_LARSEN, 2, R, 7>;
+            return launch_pdl(k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour,
+                              p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_,
+                              p.local_iters);
+        };
+        return pass_runs(L, pairs, -1) ? pick(std::true_type{}) : pick(std::false_type{});
     }
     case FAM_FH: {
         auto pick = [&](auto bf, auto run) {
