@@ -2414,8 +2414,8 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
             d.larsen_n = (float)e.pp.larsen_n; d.lim = e.pp.lim;
             d.mode = e.fam == FAM_F32 ? 0 : 1;
             d.active = 1;
-            residual_dims(e.g->L, &d.res_bx, &d.res_by);
-            res_count[i] = d.res_bx * d.res_by * e.g->nz;
+            d.ix = check_index(e.g->L, &d.res_n);
+            res_count[i] = d.res_n;
             d.res_first = (int)res_tab.size();
             d.res_slot = slots;
             slots += res_count[i];

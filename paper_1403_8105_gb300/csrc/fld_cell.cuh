@@ -271,23 +271,27 @@ __device__ __forceinline__ ff2 fast_two_sum2(float2 a, float2 b) {
     return {s, sub2(b, sub2(s, a))};
 }
 
-template <int LIM, int ROUNDS>
-__device__ __forceinline__ void cell_ff_pair(float2 p0, float2 p0lo, const float2 ps[6], const float2 ls[6],
-                                             const float2 Ds[6], float2 s_, float2 ah, float2 jj, int lim_rt,
-                                             float larsen_n, float omega, float inv2h, float floor_, int rounds_rt,
-                                             float2 &hi_new, float2 &lo_new, float2 &D_new) {
-    const int lim = LIM >= 0 ? LIM : lim_rt;
-    const int local_iters = ROUNDS > 0 ? ROUNDS : rounds_rt;
-    const float2 half = both(0.5f);
-    // the gradient (grad_floor_f)
+// FFTerms and S of two unknowns.
+struct FFTerms2 {
+    ff2 base;
+    float2 A, nA, nAlo, C;       // A.hi, and both words of A negated
+};
+
+// |grad phi|, floored (grad_floor_f of ff_terms' differences).
+__device__ __forceinline__ float2 grad_pair(const float2 ps[6], const float2 ls[6], float inv2h, float floor_) {
     const float2 gx = mul2(add2(sub2(ps[1], ps[0]), sub2(ls[1], ls[0])), both(inv2h));
     const float2 gy = mul2(add2(sub2(ps[3], ps[2]), sub2(ls[3], ls[2])), both(inv2h));
     const float2 gz = mul2(add2(sub2(ps[5], ps[4]), sub2(ls[5], ls[4])), both(inv2h));
     const float2 g2 = fma2(gx, gx, fma2(gy, gy, mul2(gz, gz)));
-    const DPoint ptx = D_point(fmaxf(sqrtf(g2.x), floor_), s_.x), pty = D_point(fmaxf(sqrtf(g2.y), floor_), s_.y);
-    // ff_terms: A = sum d_s, B = sum D_s d_s (its low word negated), C = sum D_s
-    const float2 np0 = neg2(p0);
-    float2 Ah, Al, Bh, nBl, C;
+    return make_float2(fmaxf(sqrtf(g2.x), floor_), fmaxf(sqrtf(g2.y), floor_));
+}
+
+__device__ __forceinline__ FFTerms2 ff_terms_pair(float2 p0, float2 p0lo, const float2 ps[6], const float2 ls[6],
+                                                  const float2 Ds[6], float2 ah, float2 jj) {
+    FFTerms2 T;
+    // A = sum d_s, B = sum D_s d_s (its low word negated), C = sum D_s
+    const float2 np0 = neg2(p0), half = both(0.5f);
+    float2 Ah, Al, Bh, nBl;
 #pragma unroll
     for (int s = 0; s < 6; ++s) {
         const ff2 dh = two_sum2(ps[s], np0);
@@ -298,7 +302,7 @@ __device__ __forceinline__ void cell_ff_pair(float2 p0, float2 p0lo, const float
         if (s == 0) {
             Ah = dh.hi; Al = dl;
             Bh = p; nBl = npe;
-            C = Ds[0];
+            T.C = Ds[0];
             continue;
         }
         const ff2 a = two_sum2(Ah, dh.hi);
@@ -307,36 +311,53 @@ __device__ __forceinline__ void cell_ff_pair(float2 p0, float2 p0lo, const float
         const ff2 b = two_sum2(Bh, p);
         Bh = b.hi;
         nBl = add2(nBl, sub2(npe, b.lo));
-        C = add2(C, Ds[s]);
+        T.C = add2(T.C, Ds[s]);
     }
     const float2 B = sub2(Bh, nBl);
     const float2 nBlo = add2(nBl, sub2(B, Bh));
     // base = j h^2 - sigma_a' h^2 phi + B / 2
-    ff2 base;
-    {
-        const float2 P = mul2(p0, ah);
-        const float2 e = fma2(neg2(p0lo), ah, fma2(np0, ah, P));
-        const float2 mh = sub2(e, P);
-        const float2 ml = sub2(e, add2(mh, P));
-        const ff2 t = two_sum2(mh, jj);
-        const ff2 u = fast_two_sum2(t.hi, add2(t.lo, ml));
-        const ff2 v = two_sum2(u.hi, mul2(B, half));
-        base = fast_two_sum2(v.hi, add2(v.lo, sub2(u.lo, mul2(nBlo, half))));
-    }
+    const float2 P = mul2(p0, ah);
+    const float2 e = fma2(neg2(p0lo), ah, fma2(np0, ah, P));
+    const float2 mh = sub2(e, P);
+    const float2 ml = sub2(e, add2(mh, P));
+    const ff2 t = two_sum2(mh, jj);
+    const ff2 u = fast_two_sum2(t.hi, add2(t.lo, ml));
+    const ff2 v = two_sum2(u.hi, mul2(B, half));
+    T.base = fast_two_sum2(v.hi, add2(v.lo, sub2(u.lo, mul2(nBlo, half))));
     const ff2 A = fast_two_sum2(Ah, Al);
-    const float2 nA = neg2(A.hi), nAlo = neg2(A.lo), hC = mul2(C, half);
+    T.A = A.hi;
+    T.nA = neg2(A.hi);
+    T.nAlo = neg2(A.lo);
+    return T;
+}
+
+__device__ __forceinline__ ff2 ff_S_pair(const FFTerms2 &T, float2 Dp) {
+    const float2 hd = mul2(Dp, both(0.5f));
+    const float2 p = mul2(T.A, hd);
+    const float2 ne = fma2(T.nAlo, hd, fma2(T.nA, hd, p));
+    const float2 m = sub2(p, ne);
+    const float2 nml = add2(ne, sub2(m, p));
+    const ff2 t = two_sum2(T.base.hi, m);
+    return fast_two_sum2(t.hi, add2(t.lo, sub2(T.base.lo, nml)));
+}
+
+template <int LIM, int ROUNDS>
+__device__ __forceinline__ void cell_ff_pair(float2 p0, float2 p0lo, const float2 ps[6], const float2 ls[6],
+                                             const float2 Ds[6], float2 s_, float2 ah, float2 jj, int lim_rt,
+                                             float larsen_n, float omega, float inv2h, float floor_, int rounds_rt,
+                                             float2 &hi_new, float2 &lo_new, float2 &D_new) {
+    const int lim = LIM >= 0 ? LIM : lim_rt;
+    const int local_iters = ROUNDS > 0 ? ROUNDS : rounds_rt;
+    const float2 gmax = grad_pair(ps, ls, inv2h, floor_);
+    const DPoint ptx = D_point(gmax.x, s_.x), pty = D_point(gmax.y, s_.y);
+    const FFTerms2 T = ff_terms_pair(p0, p0lo, ps, ls, Ds, ah, jj);
+    const float2 hC = mul2(T.C, both(0.5f));
     float2 delta = both(0.0f), Dp = both(0.0f);
 #pragma unroll(ROUNDS > 0 ? ROUNDS : 1)
     for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : local_iters); ++r) {
         Dp.x = D_of_f(ptx, __fadd_rn(p0.x, delta.x), floor_, lim, larsen_n);
         Dp.y = D_of_f(pty, __fadd_rn(p0.y, delta.y), floor_, lim, larsen_n);
-        const float2 hd = mul2(Dp, half);
-        const float2 p = mul2(A.hi, hd);
-        const float2 ne = fma2(nAlo, hd, fma2(nA, hd, p));
-        const float2 m = sub2(p, ne);
-        const float2 nml = add2(ne, sub2(m, p));
-        const ff2 t = two_sum2(base.hi, m);
-        const ff2 S = fast_two_sum2(t.hi, add2(t.lo, sub2(base.lo, nml)));
+        const ff2 S = ff_S_pair(T, Dp);
         const float2 num = add2(S.hi, S.lo);
         const float2 den = add2(add2(ah, mul2(Dp, both(3.0f))), hC);
         delta = make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));

@@ -155,6 +155,13 @@ cudaError_t launch_bake_march(const Layout &L, const Fields &f, float h, const d
 cudaError_t launch_validate(long long n, const Fields &f, const float *sigma_t, const float *albedo,
                             const float *j, cudaStream_t s);
 
+// Where the pairs of unknowns of a single-precision residual check lie: total =
+// pairs per half row x 2 colours x ny x nz.
+struct CheckIndex {
+    uint32_t pairs, total;
+    Divisor by_pairs, by_rows;
+};
+
 // One grid of a batched solve, read by the batched residual kernels at run
 // time (so grids can converge or change phase between checks).
 struct alignas(16) BatchDesc {
@@ -164,7 +171,8 @@ struct alignas(16) BatchDesc {
     int lim;
     int mode;            // 0: single-precision sweeps, 1: float-float correction sweeps
     int active;          // 0: converged / stopped, its CTAs return at once
-    int res_first, res_bx, res_by;      // first CTA of this grid in the residual table, grid dims
+    int res_first, res_n;               // first CTA of this grid in the residual table, number of its CTAs
+    CheckIndex ix;
     int res_slot;                       // first partial-sum slot of this grid
 };
 static_assert(sizeof(BatchDesc) % 16 == 0, "BatchDesc is read with 16-byte loads");
@@ -205,8 +213,8 @@ int multi_ctas(int nsm, int hl, int bf16, int lim, int local_iters);
 cudaError_t launch_residual_batch(const BatchDesc *descs, const int *cta_grid, int nctas, int ngrids,
                                   const int *res_count, double *partials, double *result, int lim, int margin,
                                   cudaStream_t s);
-// Pass / residual grid dimensions of a layout (CTAs = x * y * nz).
-void residual_dims(const Layout &L, int *bx, int *by);
+// Walk and number of CTAs of a layout's single-precision residual check.
+CheckIndex check_index(const Layout &L, int *ctas);
 
 // Anderson mixing of blocks of sweeps (fld_anderson.cu): m history slots of
 // g (float-float) and f (FP32) per element of the padded field, the current

@@ -857,30 +857,64 @@ __global__ void __launch_bounds__(256) k_pass_d(Layout L, const double *__restri
 // ---------------------------------------------------------------------------
 // Residual (Eq. 37) with D recomputed from the current phi.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void fresh_D_f_body(const Layout &L, const float *__restrict__ sp,
-                                               const float *__restrict__ phi, const float *__restrict__ phlo,
-                                               float *__restrict__ Df, int lim, float larsen_n, float inv2h,
-                                               float floor_, int i, int j, int k) {
-    if (i >= L.nx || j >= L.ny) return;
-    const int q = L.at(i, j, k);
-    const int xm = L.at(i - 1, j, k), xp = L.at(i + 1, j, k), ym = L.at(i, j - 1, k), yp = L.at(i, j + 1, k);
-    const int zm = L.at(i, j, k - 1), zp = L.at(i, j, k + 1);
-    float lxm = 0, lxp = 0, lym = 0, lyp = 0, lzm = 0, lzp = 0;
-    if (phlo) {
-        lxm = phlo[xm]; lxp = phlo[xp]; lym = phlo[ym]; lyp = phlo[yp];
-        lzm = phlo[zm]; lzp = phlo[zp];
+// In single precision two kernels share this walk: CTA `cta` of `ctas` takes
+// pairs of adjacent unknowns of one colour by running number (row by row, the
+// two colours of a row after one another, so both find the fields they share in
+// the caches), in strides of all CTAs.  One voxel per thread, the sums cost as
+// much as the residual itself and left one pair of partial sums per 256 voxels
+// for the last block to add: at 256^3 fresh D, residual and final sum took 104,
+// 362 and 79 us.
+constexpr int kCheckThreads = 128;
+constexpr int kCheckCtas = 1824;       // twelve per SM of 152
+
+template <typename F>
+__device__ __forceinline__ void for_pairs(const Layout &L, const CheckIndex &ix, int cta, int ctas, F &&body) {
+    for (uint32_t e = (uint32_t)cta * kCheckThreads + threadIdx.x; e < ix.total; e += (uint32_t)ctas * kCheckThreads) {
+        const uint32_t row2 = ix.by_pairs.quot(e);
+        const int t = 2 * (int)(e - row2 * ix.pairs);
+        const int c = row2 & 1;
+        const uint32_t row = row2 >> 1;
+        const int K = (int)ix.by_rows.quot(row);
+        const int J = (int)row - K * L.ny + 1;
+        Pair q;
+        pair_cells(L, c, t, J, K + 1, q);
+        if (q.first) body(q, c, t, J, K + 1);
     }
-    const float gx = __fadd_rn(__fsub_rn(phi[xp], phi[xm]), __fsub_rn(lxp, lxm));
-    const float gy = __fadd_rn(__fsub_rn(phi[yp], phi[ym]), __fsub_rn(lyp, lym));
-    const float gz = __fadd_rn(__fsub_rn(phi[zp], phi[zm]), __fsub_rn(lzp, lzm));
-    Df[q] = knudsen_D_f(gx, gy, gz, inv2h, sp[q], phi[q], floor_, lim, larsen_n);
 }
 
-__global__ void k_fresh_D_f(Layout L, const float *__restrict__ sp, const float *__restrict__ phi,
-                            const float *__restrict__ phlo, float *__restrict__ Df, int lim, float larsen_n,
-                            float inv2h, float floor_) {
-    fresh_D_f_body(L, sp, phi, phlo, Df, lim, larsen_n, inv2h, floor_, blockIdx.x * blockDim.x + threadIdx.x,
-                   blockIdx.y * blockDim.y + threadIdx.y, blockIdx.z);
+// D from the current phi (hi + lo, LO; else hi alone) at every unknown.
+template <bool LO>
+__device__ __forceinline__ void fresh_D_pairs(const Layout &L, const CheckIndex &ix, int cta, int ctas,
+                                              const float *__restrict__ sp, const float *__restrict__ phi,
+                                              const float *__restrict__ phlo, float *__restrict__ Df, int lim,
+                                              float larsen_n, float inv2h, float floor_) {
+    for_pairs(L, ix, cta, ctas, [&](const Pair &q, int, int, int, int) {
+        float2 ps[6], ls[6];
+        gather_packed(phi, q, ps);
+        if (LO) gather_packed(phlo, q, ls);
+        else
+#pragma unroll
+            for (int s = 0; s < 6; ++s) ls[s] = both(0.0f);
+        const float2 s2 = ld2(sp, q.own), p0 = ld2(phi, q.own);
+        const float2 g = grad_pair(ps, ls, inv2h, floor_);
+        const float dx = D_of_f(D_point(g.x, s2.x), p0.x, floor_, lim, larsen_n);
+        if (q.second) {
+            const float dy = D_of_f(D_point(g.y, s2.y), p0.y, floor_, lim, larsen_n);
+            *reinterpret_cast<float2 *>(Df + q.own) = make_float2(dx, dy);
+        } else {
+            Df[q.own] = dx;
+        }
+    });
+}
+
+__global__ void __launch_bounds__(kCheckThreads) k_fresh_D_f(Layout L, CheckIndex ix, const float *__restrict__ sp,
+                                                              const float *__restrict__ phi,
+                                                              const float *__restrict__ phlo, float *__restrict__ Df,
+                                                              int lim, float larsen_n, float inv2h, float floor_) {
+    if (phlo)
+        fresh_D_pairs<true>(L, ix, blockIdx.x, gridDim.x, sp, phi, phlo, Df, lim, larsen_n, inv2h, floor_);
+    else
+        fresh_D_pairs<false>(L, ix, blockIdx.x, gridDim.x, sp, phi, phlo, Df, lim, larsen_n, inv2h, floor_);
 }
 
 __global__ void k_fresh_D_d(Layout L, const double *__restrict__ sp, const double *__restrict__ phi,
@@ -895,90 +929,101 @@ __global__ void k_fresh_D_d(Layout L, const double *__restrict__ sp, const doubl
                         phi[L.at(i, j, k + 1)] - phi[L.at(i, j, k - 1)], inv2h, sp[q], phi[q], floor_, lim, larsen_n);
 }
 
-// Per-voxel residual R_p dl^2 = jh2 - ah2 phi_p + sum_s D_ps (phi_s - phi_p)
-// in float-float; its square (over the margin set) and the source square in
-// double.
-__device__ __forceinline__ void residual_f_terms(const Layout &L, const float *__restrict__ ah2,
-                                                 const float *__restrict__ jh2, const float *__restrict__ phi,
-                                                 const float *__restrict__ phlo, const float *__restrict__ Df,
-                                                 const float *__restrict__ Dghost, int margin, int i, int j, int k,
-                                                 ff &r2, ff &j2) {
+// Residual R_p dl^2 = jh2 - ah2 phi_p + sum_s D_ps (phi_s - phi_p) in
+// float-float (packed, as the correction pass forms it): per thread the sums of
+// its square over the margin set and of the source's square over all unknowns,
+// in float-float.
+template <bool LO>
+__device__ __forceinline__ void residual_pairs(const Layout &L, const CheckIndex &ix, int cta, int ctas,
+                                               const float *__restrict__ ah2, const float *__restrict__ jh2,
+                                               const float *__restrict__ phi, const float *__restrict__ phlo,
+                                               const float *__restrict__ Df, const float *__restrict__ Dghost,
+                                               int margin, ff &r2, ff &j2) {
     r2 = ff{0.0f, 0.0f};
     j2 = ff{0.0f, 0.0f};
-    if (i >= L.nx || j >= L.ny) return;
-    const int q = L.at(i, j, k);
-    const int nb[6] = {L.at(i - 1, j, k), L.at(i + 1, j, k), L.at(i, j - 1, k),
-                       L.at(i, j + 1, k), L.at(i, j, k - 1), L.at(i, j, k + 1)};
-    const bool onface[6] = {i == 0, i == L.nx - 1, j == 0, j == L.ny - 1, k == 0, k == L.nz - 1};
-    float ps[6], ls[6], Ds[6];
+    for_pairs(L, ix, cta, ctas, [&](const Pair &q, int c, int t, int J, int K) {
+        float2 ps[6], ls[6], Ds[6];
+        gather_packed(phi, q, ps);
+        if (LO) gather_packed(phlo, q, ls);
+        else
 #pragma unroll
-    for (int s = 0; s < 6; ++s) {
-        ps[s] = phi[nb[s]];
-        ls[s] = phlo ? phlo[nb[s]] : 0.0f;
+            for (int s = 0; s < 6; ++s) ls[s] = both(0.0f);
+        const int I0 = 2 * t + 2 - ((J + K + 1 + c) & 1);      // padded I of the first unknown
         // ghost neighbours keep their Dirichlet D (never recomputed)
-        Ds[s] = onface[s] ? Dghost[nb[s]] : Df[nb[s]];
-    }
-    const float ah = ah2[q];
-    const FFTerms T = ff_terms(phi[q], phlo ? phlo[q] : 0.0f, ps, ls, Ds, ah, jh2[q]);
-    const ff S = ff_S(T, Df[q]);
-    const bool in = i >= margin && i < L.nx - margin && j >= margin && j < L.ny - margin && k >= margin &&
-                    k < L.nz - margin;
-    if (in) r2 = ff_mul(S, S);
-    j2 = two_prod(jh2[q], jh2[q]);
+        const float2 xv = ld2(Df, q.xv);
+        const float xe = q.left ? (I0 == 1 ? Dghost : Df)[q.xv - 1] : (I0 + 2 == L.nx ? Dghost : Df)[q.xv + 2];
+        Ds[0] = q.left ? make_float2(xe, xv.x) : xv;
+        Ds[1] = q.left ? xv : make_float2(xv.y, xe);
+        if (I0 == L.nx) Ds[1].x = Dghost[q.left ? q.xv : q.xv + 1];
+        if (q.left && I0 + 2 == L.nx) Ds[1].y = Dghost[q.xv + 1];
+        Ds[2] = ld2(J == 1 ? Dghost : Df, q.ym);
+        Ds[3] = ld2(J == L.ny ? Dghost : Df, q.yp);
+        Ds[4] = ld2(K == 1 ? Dghost : Df, q.zm);
+        Ds[5] = ld2(K == L.nz ? Dghost : Df, q.zp);
+        const float2 jj = ld2(jh2, q.own);
+        const FFTerms2 T = ff_terms_pair(ld2(phi, q.own), LO ? ld2(phlo, q.own) : both(0.0f), ps, ls, Ds,
+                                         ld2(ah2, q.own), jj);
+        const ff2 S = ff_S_pair(T, ld2(Df, q.own));
+        const ff sx{S.hi.x, S.lo.x}, sy{S.hi.y, S.lo.y};
+        const bool in = J > margin && J <= L.ny - margin && K > margin && K <= L.nz - margin;
+        if (in && I0 > margin && I0 <= L.nx - margin) r2 = ff_add(r2, ff_mul(sx, sx));
+        j2 = ff_add(j2, two_prod(jj.x, jj.x));
+        if (q.second) {
+            if (in && I0 + 2 > margin && I0 + 2 <= L.nx - margin) r2 = ff_add(r2, ff_mul(sy, sy));
+            j2 = ff_add(j2, two_prod(jj.y, jj.y));
+        }
+    });
 }
 
-__global__ void __launch_bounds__(256) k_residual_f(Layout L, const float *__restrict__ ah2,
-                                                    const float *__restrict__ jh2, const float *__restrict__ phi,
-                                                    const float *__restrict__ phlo, const float *__restrict__ Df,
-                                                    const float *__restrict__ Dghost, int margin,
-                                                    double *__restrict__ partials) {
+// The CTA's sums into its pair of partials.
+__device__ __forceinline__ void store_partials(ff r2f, ff j2f, double *__restrict__ p) {
     __shared__ double sh[32];
-    ff r2f, j2f;
-    residual_f_terms(L, ah2, jh2, phi, phlo, Df, Dghost, margin, blockIdx.x * blockDim.x + threadIdx.x,
-                     blockIdx.y * blockDim.y + threadIdx.y, blockIdx.z, r2f, j2f);
     const double r2 = block_sum_ff(r2f, sh);
     __syncthreads();
     const double j2 = block_sum_ff(j2f, sh);
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
-        const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
-        partials[2 * b] = r2;
-        partials[2 * b + 1] = j2;
+    if (threadIdx.x == 0) {
+        p[0] = r2;
+        p[1] = j2;
     }
 }
 
-// Batched fresh D / residual / finalize: CTA b works on grid cta_grid[b] with
-// the same block decomposition as the solo launch, writes its partial sums to
-// the grid's own slots, and one block per grid sums them in the solo order.
-__global__ void __launch_bounds__(256) k_fresh_D_batch(const BatchDesc *__restrict__ descs,
-                                                       const int *__restrict__ cta_grid, int lim) {
-    const BatchDesc d = load_desc(descs + __ldg(cta_grid + blockIdx.x));
-    if (!d.active) return;
-    const int local = blockIdx.x - d.res_first;
-    const int bx = local % d.res_bx, rest = local / d.res_bx;
-    const int by = rest % d.res_by, bz = rest / d.res_by;
-    fresh_D_f_body(d.L, d.sp, d.phi, d.mode ? d.phlo : nullptr, d.Df, lim, d.larsen_n, d.inv2h, d.floor_,
-                   bx * blockDim.x + threadIdx.x, by * blockDim.y + threadIdx.y, bz);
+__global__ void __launch_bounds__(kCheckThreads) k_residual_f(Layout L, CheckIndex ix, const float *__restrict__ ah2,
+                                                               const float *__restrict__ jh2,
+                                                               const float *__restrict__ phi,
+                                                               const float *__restrict__ phlo,
+                                                               const float *__restrict__ Df,
+                                                               const float *__restrict__ Dghost, int margin,
+                                                               double *__restrict__ partials) {
+    ff r2, j2;
+    if (phlo) residual_pairs<true>(L, ix, blockIdx.x, gridDim.x, ah2, jh2, phi, phlo, Df, Dghost, margin, r2, j2);
+    else residual_pairs<false>(L, ix, blockIdx.x, gridDim.x, ah2, jh2, phi, phlo, Df, Dghost, margin, r2, j2);
+    store_partials(r2, j2, partials + 2 * (long long)blockIdx.x);
 }
 
-__global__ void __launch_bounds__(256) k_residual_batch(const BatchDesc *__restrict__ descs,
-                                                        const int *__restrict__ cta_grid, int margin,
-                                                        double *__restrict__ partials) {
-    __shared__ double sh[32];
+// Batched fresh D / residual / finalize: CTA b works on grid cta_grid[b] as CTA
+// b - res_first of the solo launch's res_n, writes its partial sums to the grid's
+// own slots, and one block per grid sums them in the solo order.
+__global__ void __launch_bounds__(kCheckThreads) k_fresh_D_batch(const BatchDesc *__restrict__ descs,
+                                                                  const int *__restrict__ cta_grid, int lim) {
     const BatchDesc d = load_desc(descs + __ldg(cta_grid + blockIdx.x));
     if (!d.active) return;
     const int local = blockIdx.x - d.res_first;
-    const int bx = local % d.res_bx, rest = local / d.res_bx;
-    const int by = rest % d.res_by, bz = rest / d.res_by;
-    ff r2f, j2f;
-    residual_f_terms(d.L, d.ah2, d.jh2, d.phi, d.mode ? d.phlo : nullptr, d.Df, d.D, margin,
-                     bx * blockDim.x + threadIdx.x, by * blockDim.y + threadIdx.y, bz, r2f, j2f);
-    const double r2 = block_sum_ff(r2f, sh);
-    __syncthreads();
-    const double j2 = block_sum_ff(j2f, sh);
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
-        partials[2 * (d.res_slot + local)] = r2;
-        partials[2 * (d.res_slot + local) + 1] = j2;
-    }
+    if (d.mode)
+        fresh_D_pairs<true>(d.L, d.ix, local, d.res_n, d.sp, d.phi, d.phlo, d.Df, lim, d.larsen_n, d.inv2h, d.floor_);
+    else
+        fresh_D_pairs<false>(d.L, d.ix, local, d.res_n, d.sp, d.phi, d.phlo, d.Df, lim, d.larsen_n, d.inv2h, d.floor_);
+}
+
+__global__ void __launch_bounds__(kCheckThreads) k_residual_batch(const BatchDesc *__restrict__ descs,
+                                                                   const int *__restrict__ cta_grid, int margin,
+                                                                   double *__restrict__ partials) {
+    const BatchDesc d = load_desc(descs + __ldg(cta_grid + blockIdx.x));
+    if (!d.active) return;
+    const int local = blockIdx.x - d.res_first;
+    ff r2, j2;
+    if (d.mode) residual_pairs<true>(d.L, d.ix, local, d.res_n, d.ah2, d.jh2, d.phi, d.phlo, d.Df, d.D, margin, r2, j2);
+    else residual_pairs<false>(d.L, d.ix, local, d.res_n, d.ah2, d.jh2, d.phi, d.phlo, d.Df, d.D, margin, r2, j2);
+    store_partials(r2, j2, partials + 2 * (long long)(d.res_slot + local));
 }
 
 __global__ void __launch_bounds__(kRedThreads) k_finalize_batch(const BatchDesc *__restrict__ descs,
@@ -1424,18 +1469,23 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
     return cudaGetLastError();
 }
 
-void residual_dims(const Layout &L, int *bx, int *by) {
-    const dim3 g = vox_grid(L);
-    *bx = (int)g.x;
-    *by = (int)g.y;
+CheckIndex check_index(const Layout &L, int *ctas) {
+    CheckIndex ix;
+    ix.pairs = (uint32_t)(((L.nx + 1) / 2 + 1) / 2);
+    ix.total = 2u * ix.pairs * (uint32_t)L.ny * (uint32_t)L.nz;
+    ix.by_pairs.set(ix.pairs);
+    ix.by_rows.set((uint32_t)L.ny);
+    const uint32_t want = (ix.total + kCheckThreads - 1) / kCheckThreads;
+    *ctas = (int)(want < (uint32_t)kCheckCtas ? want : (uint32_t)kCheckCtas);
+    return ix;
 }
 
 cudaError_t launch_residual_batch(const BatchDesc *descs, const int *cta_grid, int nctas, int ngrids,
                                   const int *res_count, double *partials, double *result, int lim, int margin,
                                   cudaStream_t s) {
     if (nctas <= 0) return cudaSuccess;
-    k_fresh_D_batch<<<nctas, vox_block(), 0, s>>>(descs, cta_grid, lim);
-    k_residual_batch<<<nctas, vox_block(), 0, s>>>(descs, cta_grid, margin, partials);
+    k_fresh_D_batch<<<nctas, kCheckThreads, 0, s>>>(descs, cta_grid, lim);
+    k_residual_batch<<<nctas, kCheckThreads, 0, s>>>(descs, cta_grid, margin, partials);
     k_finalize_batch<<<ngrids, kRedThreads, 0, s>>>(descs, res_count, partials, result);
     return cudaGetLastError();
 }
@@ -1474,8 +1524,10 @@ int reduction_blocks(const Layout &L) {
 }
 
 cudaError_t launch_fresh_D_into(const Layout &L, Fields &f, const PassParams &p, cudaStream_t s) {
-    k_fresh_D_f<<<vox_grid(L), vox_block(), 0, s>>>(L, f.sp, f.phi, nullptr, f.D, p.lim, (float)p.larsen_n,
-                                                    (float)p.inv2h, (float)p.floor_);
+    int ctas;
+    const CheckIndex ix = check_index(L, &ctas);
+    k_fresh_D_f<<<ctas, kCheckThreads, 0, s>>>(L, ix, f.sp, f.phi, nullptr, f.D, p.lim, (float)p.larsen_n,
+                                               (float)p.inv2h, (float)p.floor_);
     return cudaGetLastError();
 }
 
@@ -1490,8 +1542,10 @@ cudaError_t launch_jacobi(Family fam, const Layout &L, const Fields &f, const Pa
     } else {
         const float *src = to_second ? f.phi : f.phi2;
         float *dst = to_second ? f.phi2 : f.phi;
-        k_fresh_D_f<<<grd, blk, 0, s>>>(L, f.sp, src, nullptr, f.D, p.lim, (float)p.larsen_n, (float)p.inv2h,
-                                        (float)p.floor_);
+        int ctas;
+        const CheckIndex ix = check_index(L, &ctas);
+        k_fresh_D_f<<<ctas, kCheckThreads, 0, s>>>(L, ix, f.sp, src, nullptr, f.D, p.lim, (float)p.larsen_n,
+                                                   (float)p.inv2h, (float)p.floor_);
         k_jacobi<float><<<grd, blk, 0, s>>>(L, f.ah2, f.jh2, src, f.D, dst, (float)p.omega);
     }
     return cudaGetLastError();
@@ -1500,16 +1554,17 @@ cudaError_t launch_jacobi(Family fam, const Layout &L, const Fields &f, const Pa
 cudaError_t launch_residual(Family fam, const Layout &L, const Fields &f, const PassParams &p, int margin,
                             cudaStream_t s) {
     const dim3 grd = vox_grid(L), blk = vox_block();
-    const int nblocks = (int)(grd.x * grd.y * grd.z);
+    int nblocks = (int)(grd.x * grd.y * grd.z);
     if (nblocks > f.partial_cap) return cudaErrorInvalidValue;
     if (fam == FAM_F64) {
         k_fresh_D_d<<<grd, blk, 0, s>>>(L, f.sp64, f.phi64, f.Df64, p.lim, p.larsen_n, p.inv2h, p.floor_);
         k_residual_d<<<grd, blk, 0, s>>>(L, f.ah264, f.jh264, f.phi64, f.Df64, f.D64, margin, f.partials);
     } else {
         const float *lo = fam == FAM_F32 ? nullptr : f.phlo;
-        k_fresh_D_f<<<grd, blk, 0, s>>>(L, f.sp, f.phi, lo, f.Df, p.lim, (float)p.larsen_n, (float)p.inv2h,
-                                        (float)p.floor_);
-        k_residual_f<<<grd, blk, 0, s>>>(L, f.ah2, f.jh2, f.phi, lo, f.Df, f.D, margin, f.partials);
+        const CheckIndex ix = check_index(L, &nblocks);
+        k_fresh_D_f<<<nblocks, kCheckThreads, 0, s>>>(L, ix, f.sp, f.phi, lo, f.Df, p.lim, (float)p.larsen_n,
+                                                      (float)p.inv2h, (float)p.floor_);
+        k_residual_f<<<nblocks, kCheckThreads, 0, s>>>(L, ix, f.ah2, f.jh2, f.phi, lo, f.Df, f.D, margin, f.partials);
     }
     k_finalize<<<1, kRedThreads, 0, s>>>(f.partials, nblocks, f.result);
     return cudaGetLastError();
