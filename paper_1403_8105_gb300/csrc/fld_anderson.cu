@@ -7,8 +7,9 @@
 // (summing to 1) that minimise |sum_i a_i f_i|.  The weights come from the
 // Gram matrix <f_i, f_j>, reduced here and solved on the host.
 //
-// Per element of a padded field (both colours, ghosts and row padding
-// included -- there f is 0 and every g_i is the same value):
+// Per element of a padded field where a row has unknowns (the ghosts at its ends
+// and the padding, half of the field on a 128-voxel edge, would add f = 0 and
+// stay as they are: they are skipped):
 //   k_and_collect: g = phi (hi/lo pair, or FP64 split into one), f = g - x_cur
 //                  rounded to float, stores g in its slot (float-float) and f
 //                  (FP32), and accumulates <f, f_j> for every occupied slot j
@@ -32,6 +33,31 @@ namespace fld {
 namespace {
 
 constexpr int kAndThreads = 256;
+
+// The elements of a half row that can hold unknowns: [kXoff + 1, kXoff + 1 + half).
+struct RowSpan {
+    uint32_t hpx, half, rows;    // rows: of both colours
+    Divisor by_hpx, by_half;
+    // whether element e of a field lies in the span of its row
+    __device__ __forceinline__ bool has(uint32_t e) const {
+        return e - by_hpx.quot(e) * hpx - (kXoff + 1) < half;
+    }
+    // element v of the spans of all rows
+    __device__ __forceinline__ uint32_t at(uint32_t v) const {
+        const uint32_t r = by_half.quot(v);
+        return r * hpx + (kXoff + 1) + (v - r * half);
+    }
+};
+
+RowSpan row_span(const Layout &L) {
+    RowSpan r;
+    r.hpx = (uint32_t)L.hpx;
+    r.half = (uint32_t)(L.nx + 1) / 2;
+    r.rows = (uint32_t)(L.total / L.hpx);
+    r.by_hpx.set(r.hpx);
+    r.by_half.set(r.half);
+    return r;
+}
 
 struct SlotPtrs {
     const float2 *g[kAndersonMax];
@@ -59,17 +85,19 @@ __device__ __forceinline__ ff state_at(const float *hi, const float *lo, const d
     return ff{hi[e], lo ? lo[e] : 0.0f};
 }
 
-__global__ void __launch_bounds__(kAndThreads) k_and_capture(int n, const float *__restrict__ hi,
+__global__ void __launch_bounds__(kAndThreads) k_and_capture(RowSpan rs, const float *__restrict__ hi,
                                                               const float *__restrict__ lo,
                                                               const double *__restrict__ p64,
                                                               float2 *__restrict__ x_cur) {
-    for (long long e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    const uint32_t n = rs.rows * rs.half;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint32_t e = rs.at(i);
         const ff v = state_at(hi, lo, p64, e);
         x_cur[e] = make_float2(v.hi, v.lo);
     }
 }
 
-__global__ void __launch_bounds__(kAndThreads) k_and_collect(int n, const float *__restrict__ hi,
+__global__ void __launch_bounds__(kAndThreads) k_and_collect(int n, RowSpan rs, const float *__restrict__ hi,
                                                               const float *__restrict__ lo,
                                                               const double *__restrict__ p64,
                                                               const float2 *__restrict__ x_cur, SlotPtrs sl,
@@ -78,7 +106,8 @@ __global__ void __launch_bounds__(kAndThreads) k_and_collect(int n, const float 
     ff acc[kAndersonMax];
 #pragma unroll
     for (int j = 0; j < kAndersonMax; ++j) acc[j] = ff{0.0f, 0.0f};
-    for (long long e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < (uint32_t)n; e += gridDim.x * blockDim.x) {
+        if (!rs.has(e)) continue;
         const ff g = state_at(hi, lo, p64, e);
         const ff d = ff_sub(g, ld_ff(x_cur, e));
         const float f = __fadd_rn(d.hi, d.lo);
@@ -124,10 +153,12 @@ __global__ void __launch_bounds__(32 * kAndersonMax) k_and_reduce(const double *
     if (lane == 0) out[j] = v;
 }
 
-__global__ void __launch_bounds__(kAndThreads) k_and_mix(int n, SlotPtrs sl, int w, int s, Coef c,
+__global__ void __launch_bounds__(kAndThreads) k_and_mix(RowSpan rs, SlotPtrs sl, int w, int s, Coef c,
                                                           float *__restrict__ hi, float *__restrict__ lo,
                                                           double *__restrict__ p64, float2 *__restrict__ x_cur) {
-    for (long long e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    const uint32_t n = rs.rows * rs.half;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint32_t e = rs.at(i);
         const ff gs = ld_ff(sl.g[s], e);
         ff acc{0.0f, 0.0f};
 #pragma unroll
@@ -165,17 +196,17 @@ SlotPtrs slot_ptrs(const AndersonBuffers &b, int n, int w) {
 
 }  // namespace
 
-cudaError_t launch_anderson_capture(const AndersonBuffers &b, int n, const float *hi, const float *lo,
+cudaError_t launch_anderson_capture(const AndersonBuffers &b, const Layout &L, const float *hi, const float *lo,
                                     const double *p64, int nsm, cudaStream_t s) {
-    k_and_capture<<<and_grid(n, nsm), kAndThreads, 0, s>>>(n, hi, lo, p64, b.x);
+    k_and_capture<<<and_grid(L.total, nsm), kAndThreads, 0, s>>>(row_span(L), hi, lo, p64, b.x);
     return cudaGetLastError();
 }
 
-cudaError_t launch_anderson_collect(const AndersonBuffers &b, int n, const float *hi, const float *lo,
+cudaError_t launch_anderson_collect(const AndersonBuffers &b, const Layout &L, const float *hi, const float *lo,
                                     const double *p64, int slot, int w, int nsm, cudaStream_t s) {
-    const int nb = and_grid(n, nsm);
+    const int n = L.total, nb = and_grid(n, nsm);
     const SlotPtrs sl = slot_ptrs(b, n, w);
-    k_and_collect<<<nb, kAndThreads, 0, s>>>(n, hi, lo, p64, b.x, sl, b.g + (size_t)slot * n,
+    k_and_collect<<<nb, kAndThreads, 0, s>>>(n, row_span(L), hi, lo, p64, b.x, sl, b.g + (size_t)slot * n,
                                              b.f + (size_t)slot * n, w, slot, b.part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -183,7 +214,7 @@ cudaError_t launch_anderson_collect(const AndersonBuffers &b, int n, const float
     return cudaGetLastError();
 }
 
-cudaError_t launch_anderson_mix(const AndersonBuffers &b, int n, int slot, int w, const double *a, float *hi,
+cudaError_t launch_anderson_mix(const AndersonBuffers &b, const Layout &L, int slot, int w, const double *a, float *hi,
                                 float *lo, double *p64, int nsm, cudaStream_t s) {
     Coef c;
     for (int j = 0; j < kAndersonMax; ++j) {
@@ -191,7 +222,7 @@ cudaError_t launch_anderson_mix(const AndersonBuffers &b, int n, int slot, int w
         c.hi[j] = (float)v;
         c.lo[j] = (float)(v - (double)c.hi[j]);
     }
-    k_and_mix<<<and_grid(n, nsm), kAndThreads, 0, s>>>(n, slot_ptrs(b, n, w), w, slot, c, hi, lo, p64, b.x);
+    k_and_mix<<<and_grid(L.total, nsm), kAndThreads, 0, s>>>(row_span(L), slot_ptrs(b, L.total, w), w, slot, c, hi, lo, p64, b.x);
     return cudaGetLastError();
 }
 

@@ -941,20 +941,21 @@ fld_status preallocate(fld_grid_s *g, const fld_solve_params *p) {
     return FLD_OK;
 }
 
-// Copy the family's state into (save) or out of (restore) the snapshot.
-fld_status snapshot(fld_grid_s *g, Family fam, bool save) {
+// Copy the family's state into (save) or out of (restore) the snapshot; lo: the
+// low word of phi belongs to it (else it is zero, and is zeroed on the way back).
+fld_status snapshot(fld_grid_s *g, Family fam, bool save, bool lo) {
     const size_t nf = sizeof(float) * (size_t)g->L.total, nd = sizeof(double) * (size_t)g->L.total;
+    if (!ensure_snapshot(g, fam)) return fail(FLD_ERR_OOM, "cudaMalloc of the solve snapshot failed");
     if (fam == FAM_F64) {
-        if (!ensure_snapshot(g, fam)) return fail(FLD_ERR_OOM, "cudaMalloc of the solve snapshot failed");
         double *a[2] = {g->f.phi64, g->f.D64}, *b[2] = {g->snap_phi64, g->snap_D64};
         for (int i = 0; i < 2; ++i)
             FLD_CK(cudaMemcpyAsync(save ? b[i] : a[i], save ? a[i] : b[i], nd, cudaMemcpyDeviceToDevice, g->stream));
-    } else {
-        if (!ensure_snapshot(g, fam)) return fail(FLD_ERR_OOM, "cudaMalloc of the solve snapshot failed");
-        float *a[3] = {g->f.phi, g->f.phlo, g->f.D}, *b[3] = {g->snap_phi, g->snap_lo, g->snap_D};
-        for (int i = 0; i < 3; ++i)
-            FLD_CK(cudaMemcpyAsync(save ? b[i] : a[i], save ? a[i] : b[i], nf, cudaMemcpyDeviceToDevice, g->stream));
+        return FLD_OK;
     }
+    float *a[3] = {g->f.phi, g->f.D, g->f.phlo}, *b[3] = {g->snap_phi, g->snap_D, g->snap_lo};
+    for (int i = 0; i < (lo ? 3 : 2); ++i)
+        FLD_CK(cudaMemcpyAsync(save ? b[i] : a[i], save ? a[i] : b[i], nf, cudaMemcpyDeviceToDevice, g->stream));
+    if (!lo && !save && g->lo_live) FLD_CK(cudaMemsetAsync(g->f.phlo, 0, nf, g->stream));
     return FLD_OK;
 }
 
@@ -1469,16 +1470,18 @@ fld_status fld_set_state(fld_grid g, const double *phi, const double *D, int whe
     // Both families receive the values, so an FP64 continuation keeps them
     // exactly (the float family rounds D to float).
     if ((st = ensure_f64(g)) != FLD_OK) return st;
-    if (!g->valid_float && !g->valid_d) {
+    // (a field that is given is overwritten whole, ghosts included)
+    if (phi && D) {
+    } else if (!g->valid_float && !g->valid_d) {
         // a partial update of a grid without state: start from zeros
         FLD_CK(launch_init_f(g->L, g->f.phi, g->f.phlo, g->f.D, 0.0, 0.0, 0.0, 0.0, g->stream));
         FLD_CK(launch_init_d(g->L, g->f.phi64, g->f.D64, 0.0, 0.0, 0.0, 0.0, g->stream));
     } else if (g->valid_d && !g->valid_float) {
-        FLD_CK(launch_d_to_f(g->L, g->f.phi64, g->f.phi, g->f.phlo, g->stream));
-        FLD_CK(launch_d_to_f(g->L, g->f.D64, g->f.D, nullptr, g->stream));
+        if (!phi) FLD_CK(launch_d_to_f(g->L, g->f.phi64, g->f.phi, g->f.phlo, g->stream));
+        if (!D) FLD_CK(launch_d_to_f(g->L, g->f.D64, g->f.D, nullptr, g->stream));
     } else if (g->valid_float && !g->valid_d) {
-        FLD_CK(launch_f_to_d(g->L, g->f.phi, g->lo_live ? g->f.phlo : nullptr, g->f.phi64, g->stream));
-        FLD_CK(launch_f_to_d(g->L, g->f.D, nullptr, g->f.D64, g->stream));
+        if (!phi) FLD_CK(launch_f_to_d(g->L, g->f.phi, g->lo_live ? g->f.phlo : nullptr, g->f.phi64, g->stream));
+        if (!D) FLD_CK(launch_f_to_d(g->L, g->f.D, nullptr, g->f.D64, g->stream));
     }
     double *stage = nullptr;
     if (where != FLD_MEM_DEVICE) FLD_CK(cudaMalloc((void **)&stage, sizeof(double) * n));
@@ -1494,9 +1497,8 @@ fld_status fld_set_state(fld_grid g, const double *phi, const double *D, int whe
             }
             src = stage;
         }
-        cudaError_t e = a == 0 ? launch_unpack_to_f(g->L, src, g->f.phi, g->f.phlo, g->stream)
-                               : launch_unpack_to_f(g->L, src, g->f.D, nullptr, g->stream);
-        if (e == cudaSuccess) e = launch_unpack_to_d(g->L, src, a == 0 ? g->f.phi64 : g->f.D64, g->stream);
+        cudaError_t e = a == 0 ? launch_unpack(g->L, src, g->f.phi, g->f.phlo, g->f.phi64, g->stream)
+                               : launch_unpack(g->L, src, g->f.D, nullptr, g->f.D64, g->stream);
         if (e != cudaSuccess) {
             if (stage) cudaFree(stage);
             return cuda_fail(e, "unpack state");
@@ -1729,7 +1731,7 @@ fld_status solve_core(fld_grid g, const fld_solve_params *p, fld_solve_result *r
     Family snap_fam = fam;
     bool snap_lo_live = g->lo_live;
     auto save = [&]() -> fld_status {
-        fld_status s2 = snapshot(g, fam, true);
+        fld_status s2 = snapshot(g, fam, true, g->lo_live);
         snap_fam = fam;
         snap_lo_live = g->lo_live;
         return s2;
@@ -1787,7 +1789,7 @@ fld_status solve_core(fld_grid g, const fld_solve_params *p, fld_solve_result *r
             float *hi, *lo;
             double *p64;
             state_ptrs(&hi, &lo, &p64);
-            FLD_CK(launch_anderson_capture(g->anderson, g->L.total, hi, lo, p64, g->nsm, g->stream));
+            FLD_CK(launch_anderson_capture(g->anderson, g->L, hi, lo, p64, g->nsm, g->stream));
             g->kernels += 1;
             have_x = true;
             acount = 0;
@@ -1820,7 +1822,7 @@ fld_status solve_core(fld_grid g, const fld_solve_params *p, fld_solve_result *r
             if (am > 1 && !mix_off && it < p->max_iters) {
                 // the mixed iteration stalled above tol: continue with plain
                 // sweeps (and the plain solve's windows) from the best state
-                if ((st = snapshot(g, snap_fam, false)) != FLD_OK) return st;
+                if ((st = snapshot(g, snap_fam, false, snap_lo_live)) != FLD_OK) return st;
                 fam = snap_fam;
                 ctl.fam = fam;
                 set_valid(g, fam);
@@ -1836,11 +1838,11 @@ fld_status solve_core(fld_grid g, const fld_solve_params *p, fld_solve_result *r
                 stalled = true;
             }
             break;
-        case ACT_SAVE:
-            if ((st = save()) != FLD_OK) return st;
+        case ACT_SAVE:   // (after the last block nothing returns to it)
+            if (it < p->max_iters && (st = save()) != FLD_OK) return st;
             break;
         case ACT_RESTORE:
-            if ((st = snapshot(g, snap_fam, false)) != FLD_OK) return st;
+            if ((st = snapshot(g, snap_fam, false, snap_lo_live)) != FLD_OK) return st;
             fam = snap_fam;
             ctl.fam = fam;
             set_valid(g, fam);
@@ -1868,7 +1870,7 @@ fld_status solve_core(fld_grid g, const fld_solve_params *p, fld_solve_result *r
             float *hi, *lo;
             double *p64;
             state_ptrs(&hi, &lo, &p64);
-            FLD_CK(launch_anderson_collect(g->anderson, g->L.total, hi, lo, p64, slot, w, g->nsm, g->stream));
+            FLD_CK(launch_anderson_collect(g->anderson, g->L, hi, lo, p64, slot, w, g->nsm, g->stream));
             double dots[kAndersonMax];
             FLD_CK(cudaMemcpyAsync(dots, g->anderson.dots, sizeof(double) * w, cudaMemcpyDeviceToHost, g->stream));
             FLD_CK(cudaStreamSynchronize(g->stream));
@@ -1879,7 +1881,7 @@ fld_status solve_core(fld_grid g, const fld_solve_params *p, fld_solve_result *r
             if (w == 1) wts[0] = 1.0;   // x = g: the next block starts where this one ended
             else ok = anderson_weights(gram, w, wts);
             if (ok) {
-                FLD_CK(launch_anderson_mix(g->anderson, g->L.total, slot, w, wts, hi, lo, p64, g->nsm, g->stream));
+                FLD_CK(launch_anderson_mix(g->anderson, g->L, slot, w, wts, hi, lo, p64, g->nsm, g->stream));
                 g->kernels += 1;
                 if (w > 1) ++res.anderson_steps;
             } else {
@@ -2249,7 +2251,7 @@ fld_status fld_server_add(fld_server s, fld_grid g, long long tag) {
         }
     }
     if (a == ACT_SAVE) {
-        if ((st = snapshot(g, e.fam, true)) != FLD_OK) return st;
+        if ((st = snapshot(g, e.fam, true, g->lo_live)) != FLD_OK) return st;
         e.snap_fam = e.fam;
         e.snap_lo = g->lo_live;
     }
@@ -2357,7 +2359,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
                 float *hi, *lo;
                 double *p64;
                 anderson_state(e.g, e.fam, &hi, &lo, &p64);
-                const cudaError_t ce = launch_anderson_capture(e.g->anderson, e.g->L.total, hi, lo, p64, e.g->nsm,
+                const cudaError_t ce = launch_anderson_capture(e.g->anderson, e.g->L, hi, lo, p64, e.g->nsm,
                                                                e.g->stream);
                 if (ce != cudaSuccess) {
                     e.g->stream = s->bs;
@@ -2470,7 +2472,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
             case ACT_STALLED:
                 if (e.am > 1 && !e.mix_off && e.res.iterations < p->max_iters) {
                     // as fld_solve: plain sweeps from the best state
-                    if ((st = snapshot(g, e.snap_fam, false)) != FLD_OK) return st;
+                    if ((st = snapshot(g, e.snap_fam, false, e.snap_lo)) != FLD_OK) return st;
                     e.fam = e.snap_fam;
                     e.ctl.fam = e.fam;
                     set_valid(g, e.fam);
@@ -2488,12 +2490,12 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
                 }
                 break;
             case ACT_SAVE:
-                if ((st = snapshot(g, e.fam, true)) != FLD_OK) return st;
+                if ((st = snapshot(g, e.fam, true, g->lo_live)) != FLD_OK) return st;
                 e.snap_fam = e.fam;
                 e.snap_lo = g->lo_live;
                 break;
             case ACT_RESTORE:
-                if ((st = snapshot(g, e.snap_fam, false)) != FLD_OK) return st;
+                if ((st = snapshot(g, e.snap_fam, false, e.snap_lo)) != FLD_OK) return st;
                 e.fam = e.snap_fam;
                 e.ctl.fam = e.fam;
                 set_valid(g, e.fam);
@@ -2528,7 +2530,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
             float *hi, *lo;
             double *p64;
             anderson_state(e.g, e.fam, &hi, &lo, &p64);
-            FLD_CK(launch_anderson_collect(e.g->anderson, e.g->L.total, hi, lo, p64, slot, w, e.g->nsm, s->bs));
+            FLD_CK(launch_anderson_collect(e.g->anderson, e.g->L, hi, lo, p64, slot, w, e.g->nsm, s->bs));
             FLD_CK(cudaMemcpyAsync(&dots[i * kAndersonMax], e.g->anderson.dots, sizeof(double) * w,
                                    cudaMemcpyDeviceToHost, s->bs));
             s->launches += 2;
@@ -2550,7 +2552,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
                 float *hi, *lo;
                 double *p64;
                 anderson_state(e.g, e.fam, &hi, &lo, &p64);
-                FLD_CK(launch_anderson_mix(e.g->anderson, e.g->L.total, slot, w, wts, hi, lo, p64, e.g->nsm, s->bs));
+                FLD_CK(launch_anderson_mix(e.g->anderson, e.g->L, slot, w, wts, hi, lo, p64, e.g->nsm, s->bs));
                 s->launches += 1;
                 if (w > 1) ++e.res.anderson_steps;
             } else {

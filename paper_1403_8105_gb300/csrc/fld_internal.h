@@ -121,8 +121,8 @@ cudaError_t launch_init_d(const Layout &L, double *phi, double *D, double phi0, 
 
 // Conversions between the packed (nx+2)(ny+2)(nz+2) double layout and the
 // device fields.  dst_lo may be null (single float); src_lo likewise.
-cudaError_t launch_unpack_to_f(const Layout &L, const double *src, float *dst_hi, float *dst_lo, cudaStream_t s);
-cudaError_t launch_unpack_to_d(const Layout &L, const double *src, double *dst, cudaStream_t s);
+cudaError_t launch_unpack(const Layout &L, const double *src, float *dst_hi, float *dst_lo, double *dst,
+                          cudaStream_t s);
 cudaError_t launch_pack_from_f(const Layout &L, const float *hi, const float *lo, double *dst, cudaStream_t s);
 cudaError_t launch_pack_from_d(const Layout &L, const double *src, double *dst, cudaStream_t s);
 // Between families (float-float <-> double) in the device layout.
@@ -228,13 +228,13 @@ struct AndersonBuffers {
     double *dots = nullptr;   // kAndersonMax
 };
 // x = the current state (hi + lo, hi alone when lo is null, or p64).
-cudaError_t launch_anderson_capture(const AndersonBuffers &b, int n, const float *hi, const float *lo,
+cudaError_t launch_anderson_capture(const AndersonBuffers &b, const Layout &L, const float *hi, const float *lo,
                                     const double *p64, int nsm, cudaStream_t s);
 // g -> slot, f = g - x -> slot, dots[j] = <f, f_j> for the w occupied slots.
-cudaError_t launch_anderson_collect(const AndersonBuffers &b, int n, const float *hi, const float *lo,
+cudaError_t launch_anderson_collect(const AndersonBuffers &b, const Layout &L, const float *hi, const float *lo,
                                     const double *p64, int slot, int w, int nsm, cudaStream_t s);
 // state = x = g_slot + sum_{j != slot} a_j (g_j - g_slot).
-cudaError_t launch_anderson_mix(const AndersonBuffers &b, int n, int slot, int w, const double *a, float *hi,
+cudaError_t launch_anderson_mix(const AndersonBuffers &b, const Layout &L, int slot, int w, const double *a, float *hi,
                                 float *lo, double *p64, int nsm, cudaStream_t s);
 
 // Temporally blocked red-black sweeps (fld_tiled.cu).  Configuration ids
