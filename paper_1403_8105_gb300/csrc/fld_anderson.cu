@@ -97,25 +97,46 @@ __global__ void __launch_bounds__(kAndThreads) k_and_capture(RowSpan rs, const f
     }
 }
 
+// W: slots the sums have room for (w <= W).  Each thread's elements are added in
+// order, two of them loaded at a time: the loads, not the sums, take the time
+// (128^3, w = 8: 74 -> 31 us a launch).
+template <int W>
 __global__ void __launch_bounds__(kAndThreads) k_and_collect(int n, RowSpan rs, const float *__restrict__ hi,
                                                               const float *__restrict__ lo,
                                                               const double *__restrict__ p64,
                                                               const float2 *__restrict__ x_cur, SlotPtrs sl,
                                                               float2 *__restrict__ g_out, float *__restrict__ f_out,
                                                               int w, int s, double *__restrict__ part) {
-    ff acc[kAndersonMax];
+    constexpr int U = 2;
+    ff acc[W];
 #pragma unroll
-    for (int j = 0; j < kAndersonMax; ++j) acc[j] = ff{0.0f, 0.0f};
-    for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < (uint32_t)n; e += gridDim.x * blockDim.x) {
-        if (!rs.has(e)) continue;
-        const ff g = state_at(hi, lo, p64, e);
-        const ff d = ff_sub(g, ld_ff(x_cur, e));
-        const float f = __fadd_rn(d.hi, d.lo);
-        g_out[e] = make_float2(g.hi, g.lo);
-        f_out[e] = f;
+    for (int j = 0; j < W; ++j) acc[j] = ff{0.0f, 0.0f};
+    const uint32_t stride = gridDim.x * blockDim.x;
+    for (uint32_t e0 = blockIdx.x * blockDim.x + threadIdx.x; e0 < (uint32_t)n; e0 += U * stride) {
+        ff g[U], x[U];
+        float fj[U][W];
+        bool on[U];
 #pragma unroll
-        for (int j = 0; j < kAndersonMax; ++j) {
-            if (j < w) acc[j] = ff_add(acc[j], two_prod(f, j == s ? f : sl.f[j][e]));
+        for (int u = 0; u < U; ++u) {
+            const uint32_t e = e0 + u * stride;
+            on[u] = e < (uint32_t)n && rs.has(e);
+            if (!on[u]) continue;
+            g[u] = state_at(hi, lo, p64, e);
+            x[u] = ld_ff(x_cur, e);
+#pragma unroll
+            for (int j = 0; j < W; ++j) fj[u][j] = j < w && j != s ? sl.f[j][e] : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (!on[u]) continue;
+            const uint32_t e = e0 + u * stride;
+            const ff d = ff_sub(g[u], x[u]);
+            const float f = __fadd_rn(d.hi, d.lo);
+            g_out[e] = make_float2(g[u].hi, g[u].lo);
+            f_out[e] = f;
+#pragma unroll
+            for (int j = 0; j < W; ++j)
+                if (j < w) acc[j] = ff_add(acc[j], two_prod(f, j == s ? f : fj[u][j]));
         }
     }
     // block reduction of every accumulator: float-float warp shuffles, then
@@ -124,7 +145,7 @@ __global__ void __launch_bounds__(kAndThreads) k_and_collect(int n, RowSpan rs, 
     __shared__ double red[kAndThreads / 32][kAndersonMax];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int j = 0; j < kAndersonMax; ++j) {
+    for (int j = 0; j < W; ++j) {
         if (j >= w) break;
         ff v = acc[j];
         for (int o = 16; o > 0; o >>= 1) {
@@ -206,7 +227,8 @@ cudaError_t launch_anderson_collect(const AndersonBuffers &b, const Layout &L, c
                                     const double *p64, int slot, int w, int nsm, cudaStream_t s) {
     const int n = L.total, nb = and_grid(n, nsm);
     const SlotPtrs sl = slot_ptrs(b, n, w);
-    k_and_collect<<<nb, kAndThreads, 0, s>>>(n, row_span(L), hi, lo, p64, b.x, sl, b.g + (size_t)slot * n,
+    auto k = w <= 4 ? k_and_collect<4> : w <= 8 ? k_and_collect<8> : k_and_collect<kAndersonMax>;
+    k<<<nb, kAndThreads, 0, s>>>(n, row_span(L), hi, lo, p64, b.x, sl, b.g + (size_t)slot * n,
                                              b.f + (size_t)slot * n, w, slot, b.part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
