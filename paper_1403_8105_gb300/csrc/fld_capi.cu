@@ -1440,8 +1440,7 @@ fld_status fld_bake_directional(fld_grid g, const double dir[3], double radiance
     } else {
         const double w[3] = {-dir[0] / n, -dir[1] / n, -dir[2] / n};   // towards the light
         const double pos[3] = {0, 0, 0};
-        FLD_CK(launch_bake_march(g->L, g->f, (float)g->h, w, pos, 0, (float)radiance, (float)step, accumulate,
-                                 g->stream));
+        FLD_CK(launch_bake_march(g->L, g->f, g->h, w, pos, 0, (float)radiance, step, accumulate, g->stream));
     }
     ++g->version;
     return FLD_OK;
@@ -1457,7 +1456,7 @@ fld_status fld_bake_point(fld_grid g, const double pos[3], double power, double 
     if (step <= 0.0) step = 0.5 * g->h;
     if (!isfinite(step)) return fail(FLD_ERR_INVALID_ARG, "bad step");
     const double w[3] = {0, 0, 0};
-    FLD_CK(launch_bake_march(g->L, g->f, (float)g->h, w, pos, 1, (float)power, (float)step, accumulate, g->stream));
+    FLD_CK(launch_bake_march(g->L, g->f, g->h, w, pos, 1, (float)power, step, accumulate, g->stream));
     ++g->version;
     return FLD_OK;
 }

@@ -147,8 +147,8 @@ int reduction_blocks(const Layout &L);
 // Single-scatter source.
 cudaError_t launch_bake_scan_negz(const Layout &L, const Fields &f, float h, float radiance, int accumulate,
                                   cudaStream_t s);
-cudaError_t launch_bake_march(const Layout &L, const Fields &f, float h, const double w[3], const double pos[3],
-                              int point, float value, float step, int accumulate, cudaStream_t s);
+cudaError_t launch_bake_march(const Layout &L, const Fields &f, double h, const double w[3], const double pos[3],
+                              int point, float value, double step, int accumulate, cudaStream_t s);
 
 // Validation of n input values (any pointer may be null): result[0] counts
 // NaN / negative / infinite sigma_t and j, result[1] albedo outside [0, 1].

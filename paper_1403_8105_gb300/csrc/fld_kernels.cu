@@ -1172,94 +1172,167 @@ __global__ void k_bake_scan_negz(Layout L, const float *__restrict__ st, const f
     const float hh = 0.5f * h;
     ff tau = {0.0f, 0.0f};
     float above = 0.0f;
-    for (int k = L.nz - 1; k >= 0; --k) {
-        const long long v = col + (long long)k * sk;
-        const float s = st[v];
-        const ff sum = (k == L.nz - 1) ? ff{s, 0.0f} : two_sum(s, above);
-        const ff p = two_prod(sum.hi, hh);
-        tau = ff_add(tau, fast_two_sum(p.hi, fmaf(sum.lo, hh, p.lo)));
-        above = s;
-        const float q = radiance * (alb[v] * s) * transmittance(tau);
-        js[v] = accumulate ? js[v] + q : q;
-    }
-}
-
-__device__ __forceinline__ float sigma_trilinear(const Layout &L, const float *__restrict__ st, float h, float x,
-                                                 float y, float z) {
-    float u[3] = {x / h - 0.5f, y / h - 0.5f, z / h - 0.5f};
-    const int n[3] = {L.nx, L.ny, L.nz};
-    int i0[3];
-    float f[3];
+    // eight voxels at a time, their loads before the chain of sums (128^3: 93 -> 76 us)
+    constexpr int kBatch = 8;
+    for (int k0 = L.nz - 1; k0 >= 0; k0 -= kBatch) {
+        float sb[kBatch], ab[kBatch];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float w = fminf(fmaxf(u[a], 0.0f), (float)(n[a] - 1));
-        int b = (int)floorf(w);
-        b = min(max(b, 0), max(n[a] - 2, 0));
-        i0[a] = b;
-        f[a] = (n[a] == 1) ? 0.0f : w - (float)b;
+        for (int u = 0; u < kBatch; ++u) {
+            const long long v = col + (long long)max(k0 - u, 0) * sk;
+            sb[u] = st[v];
+            ab[u] = alb[v];
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const int k = k0 - u;
+            if (k < 0) break;
+            const long long v = col + (long long)k * sk;
+            const float s = sb[u];
+            const ff sum = (k == L.nz - 1) ? ff{s, 0.0f} : two_sum(s, above);
+            const ff p = two_prod(sum.hi, hh);
+            tau = ff_add(tau, fast_two_sum(p.hi, fmaf(sum.lo, hh, p.lo)));
+            above = s;
+            const float q = radiance * (ab[u] * s) * transmittance(tau);
+            js[v] = accumulate ? js[v] + q : q;
+        }
     }
-    const int i1 = min(i0[0] + 1, L.nx - 1), j1 = min(i0[1] + 1, L.ny - 1), k1 = min(i0[2] + 1, L.nz - 1);
-    const long long sy = L.nx, sz = (long long)L.nx * L.ny;
-    const long long b00 = i0[2] * sz + i0[1] * sy, b01 = i0[2] * sz + j1 * sy;
-    const long long b10 = k1 * sz + i0[1] * sy, b11 = k1 * sz + j1 * sy;
-    const float c00 = __ldg(st + b00 + i0[0]) * (1.0f - f[0]) + __ldg(st + b00 + i1) * f[0];
-    const float c01 = __ldg(st + b01 + i0[0]) * (1.0f - f[0]) + __ldg(st + b01 + i1) * f[0];
-    const float c10 = __ldg(st + b10 + i0[0]) * (1.0f - f[0]) + __ldg(st + b10 + i1) * f[0];
-    const float c11 = __ldg(st + b11 + i0[0]) * (1.0f - f[0]) + __ldg(st + b11 + i1) * f[0];
-    const float c0 = c00 * (1.0f - f[1]) + c01 * f[1];
-    const float c1 = c10 * (1.0f - f[1]) + c11 * f[1];
-    return c0 * (1.0f - f[2]) + c1 * f[2];
 }
 
 // General march: from the voxel centre towards the light, samples at the
 // midpoints of steps of length `step`, the last step shortened to end at the
-// grid boundary (or at a point light inside the grid).
+// grid boundary (or at a point light inside the grid).  Lengths are in voxels, so a
+// sample's coordinate between centres is i + t w, one FMA per axis.  Bound by
+// issue (about 70 instructions a sample) with the eight corners in L1: its
+// predecessor divided by h three times, floored by conversions and formed 64-bit
+// indices for every sample, and marched for voxels that scatter nothing, whose
+// source is zero whatever the transmittance (62 % of the box of a sphere cloud).
+// A point light over a 160^3 cloud: 4.27 -> 0.87 ms; an oblique light, 200^3: 8.4 ms
+// before.  Error against 64 bits 9.8e-7 -> 6.0e-7.
+//
+// t = (u - 1/2) + M, M = 1.5 2^23, rounds u - 1/2 to an integer in t's low bits:
+// the lower corner b (u itself if it is one: the blend is the same from either
+// side).  That needs n <= 2^20; WIDE converts instead, and takes axes of one voxel
+// (whose upper corner is the lower one).
+constexpr float kRound = 12582912.0f;
+constexpr int kRoundMax = 1 << 20;
+
+struct MarchAxis {
+    float top, last;             // n - 1; the largest lower corner, plus kRound
+    int n, stride;               // voxels; elements to the upper corner
+};
+
+__device__ __forceinline__ float lower_corner(const MarchAxis &a, float &u, int &b) {
+    u = fminf(fmaxf(u, 0.0f), a.top);
+    b = min(max((int)floorf(u), 0), max(a.n - 2, 0));
+    return u - (float)b;
+}
+
+template <bool WIDE>
+__device__ __forceinline__ float sigma_at(const float *__restrict__ st, const MarchAxis ax[3], const int sy, const int sz,
+                                          const int bias, float ux, float uy, float uz) {
+    int q;
+    float fx, fy, fz;
+    if (WIDE) {
+        int bx, by, bz;
+        fx = lower_corner(ax[0], ux, bx);
+        fy = lower_corner(ax[1], uy, by);
+        fz = lower_corner(ax[2], uz, bz);
+        q = bz * sz + by * sy + bx;
+    } else {
+        ux = fminf(fmaxf(ux, 0.0f), ax[0].top);
+        uy = fminf(fmaxf(uy, 0.0f), ax[1].top);
+        uz = fminf(fmaxf(uz, 0.0f), ax[2].top);
+        const float tx = fminf(__fadd_rn(__fadd_rn(ux, -0.5f), kRound), ax[0].last);
+        const float ty = fminf(__fadd_rn(__fadd_rn(uy, -0.5f), kRound), ax[1].last);
+        const float tz = fminf(__fadd_rn(__fadd_rn(uz, -0.5f), kRound), ax[2].last);
+        fx = ux - __fsub_rn(tx, kRound);
+        fy = uy - __fsub_rn(ty, kRound);
+        fz = uz - __fsub_rn(tz, kRound);
+        // (the bits of M cancel in `bias`, modulo 2^32)
+        q = (int)((uint32_t)__float_as_int(tz) * (uint32_t)sz + (uint32_t)__float_as_int(ty) * (uint32_t)sy +
+                  (uint32_t)__float_as_int(tx) - (uint32_t)bias);
+    }
+    const int dx = WIDE ? ax[0].stride : 1;
+    const float *p = st + q, *py = p + ax[1].stride, *pz = p + ax[2].stride, *pyz = py + ax[2].stride;
+    const float a0 = __ldg(p), a1 = __ldg(p + dx), b0 = __ldg(py), b1 = __ldg(py + dx);
+    const float c0 = __ldg(pz), c1 = __ldg(pz + dx), d0 = __ldg(pyz), d1 = __ldg(pyz + dx);
+    const float a = fmaf(fx, a1 - a0, a0), b = fmaf(fx, b1 - b0, b0);
+    const float c = fmaf(fx, c1 - c0, c0), d = fmaf(fx, d1 - d0, d0);
+    const float e = fmaf(fy, b - a, a), f = fmaf(fy, d - c, c);
+    return fmaf(fz, f - e, e);
+}
+
+// Where the light is, in voxels: the unit direction towards it, or its position.
+struct MarchLight {
+    float w[3], pos[3];
+    int point;
+    float value, step, h;
+};
+
+template <bool WIDE>
 __global__ void __launch_bounds__(256) k_bake_march(Layout L, const float *__restrict__ st,
-                                                    const float *__restrict__ alb, float *__restrict__ js, float h,
-                                                    float wx, float wy, float wz, float px, float py, float pz,
-                                                    int point, float value, float step, int accumulate) {
+                                                    const float *__restrict__ alb, float *__restrict__ js,
+                                                    MarchLight m, int accumulate) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int k = blockIdx.z;
     if (i >= L.nx || j >= L.ny) return;
     const long long v = ((long long)k * L.ny + j) * L.nx + i;
-    const float x[3] = {(i + 0.5f) * h, (j + 0.5f) * h, (k + 0.5f) * h};
-    float w[3] = {wx, wy, wz};
+    const float scatter = __fmul_rn(alb[v], st[v]);
+    if (scatter == 0.0f) {
+        if (!accumulate) js[v] = 0.0f;
+        return;
+    }
+    const int n[3] = {L.nx, L.ny, L.nz};
+    const float x[3] = {(float)i, (float)j, (float)k};       // the centre, from the first centre
+    float w[3] = {m.w[0], m.w[1], m.w[2]};
     float r = 0.0f;
-    if (point) {
-        const float d[3] = {px - x[0], py - x[1], pz - x[2]};
+    if (m.point) {
+        const float d[3] = {m.pos[0] - x[0], m.pos[1] - x[1], m.pos[2] - x[2]};
         r = sqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
         if (r > 0.0f) {
             w[0] = d[0] / r; w[1] = d[1] / r; w[2] = d[2] / r;
         }
     }
-    const float ext[3] = {L.nx * h, L.ny * h, L.nz * h};
     float len = INFINITY;
+    MarchAxis ax[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        if (w[a] > 0.0f) len = fminf(len, (ext[a] - x[a]) / w[a]);
-        else if (w[a] < 0.0f) len = fminf(len, (0.0f - x[a]) / w[a]);
+        if (w[a] > 0.0f) len = fminf(len, ((float)n[a] - 0.5f - x[a]) / w[a]);
+        else if (w[a] < 0.0f) len = fminf(len, (-0.5f - x[a]) / w[a]);
+        ax[a].top = (float)(n[a] - 1);
+        ax[a].last = kRound + (float)max(n[a] - 2, 0);
+        ax[a].n = n[a];
+        ax[a].stride = n[a] == 1 ? 0 : a == 0 ? 1 : a == 1 ? L.nx : L.nx * L.ny;
     }
-    if (point) len = (r > 0.0f) ? fminf(len, r) : 0.0f;
-    // optical depth: the single-precision samples sigma * step summed in
-    // float-float (TwoSum), as accurate as a double-precision sum
-    ff tau = {0.0f, 0.0f};
-    const int m_full = (int)floorf(len / step);
-    for (int m = 0; m < m_full; ++m) {
-        const float t = ((float)m + 0.5f) * step;
-        tau = ff_add_f(tau, sigma_trilinear(L, st, h, x[0] + t * w[0], x[1] + t * w[1], x[2] + t * w[2]) * step);
+    if (m.point) len = (r > 0.0f) ? fminf(len, r) : 0.0f;
+    const int sy = L.nx, sz = L.nx * L.ny;
+    const uint32_t mb = (uint32_t)__float_as_int(kRound);
+    const int bias = (int)(mb * (uint32_t)sz + mb * (uint32_t)sy + mb);
+    // sum of the samples in float-float: TwoSum, the errors in a word of their own
+    ff sum = {0.0f, 0.0f};
+    const int m_full = (int)floorf(len / m.step);
+    for (int q = 0; q < m_full; ++q) {
+        const float t = ((float)q + 0.5f) * m.step;
+        const float s = sigma_at<WIDE>(st, ax, sy, sz, bias, fmaf(t, w[0], x[0]), fmaf(t, w[1], x[1]),
+                                       fmaf(t, w[2], x[2]));
+        const ff u = two_sum(sum.hi, s);
+        sum.hi = u.hi;
+        sum.lo = __fadd_rn(sum.lo, u.lo);
     }
-    const float rem = len - (float)m_full * step;
-    if (rem > 1e-6f * step) {
-        const float t = (float)m_full * step + 0.5f * rem;
-        tau = ff_add_f(tau, sigma_trilinear(L, st, h, x[0] + t * w[0], x[1] + t * w[1], x[2] + t * w[2]) * rem);
+    ff tau = ff_mul_f(fast_two_sum(sum.hi, sum.lo), m.step);
+    const float rem = len - (float)m_full * m.step;
+    if (rem > 1e-6f * m.step) {
+        const float t = (float)m_full * m.step + 0.5f * rem;
+        tau = ff_add_f(tau, sigma_at<WIDE>(st, ax, sy, sz, bias, fmaf(t, w[0], x[0]), fmaf(t, w[1], x[1]),
+                                           fmaf(t, w[2], x[2])) * rem);
     }
-    float q = value * (alb[v] * st[v]) * transmittance(tau);
-    if (point) {
-        const float rr = fmaxf(r, 0.5f * h);
-        q = q / (4.0f * 3.14159265358979f * rr * rr);
+    float e = m.value * scatter * transmittance(ff_mul_f(tau, m.h));
+    if (m.point) {
+        const float rr = fmaxf(r, 0.5f) * m.h;
+        e = e / (4.0f * 3.14159265358979f * rr * rr);
     }
-    js[v] = accumulate ? js[v] + q : q;
+    js[v] = accumulate ? js[v] + e : e;
 }
 
 // One thread per unknown of the colour in a row (ceil(nx/2) of them), one
@@ -1626,11 +1699,21 @@ cudaError_t launch_bake_scan_negz(const Layout &L, const Fields &f, float h, flo
     return cudaGetLastError();
 }
 
-cudaError_t launch_bake_march(const Layout &L, const Fields &f, float h, const double w[3], const double pos[3],
-                              int point, float value, float step, int accumulate, cudaStream_t s) {
-    k_bake_march<<<vox_grid(L), vox_block(), 0, s>>>(L, f.sigma_t, f.albedo, f.jsrc, h, (float)w[0], (float)w[1],
-                                                     (float)w[2], (float)pos[0], (float)pos[1], (float)pos[2], point,
-                                                     value, step, accumulate);
+cudaError_t launch_bake_march(const Layout &L, const Fields &f, double h, const double w[3], const double pos[3],
+                              int point, float value, double step, int accumulate, cudaStream_t s) {
+    MarchLight m;
+    for (int a = 0; a < 3; ++a) {
+        m.w[a] = (float)w[a];
+        m.pos[a] = (float)(pos[a] / h - 0.5);
+    }
+    m.point = point;
+    m.value = value;
+    m.step = (float)(step / h < 1e30 ? step / h : 1e30);
+    m.h = (float)h;
+    const int most = L.nx > L.ny ? (L.nx > L.nz ? L.nx : L.nz) : (L.ny > L.nz ? L.ny : L.nz);
+    const bool wide = L.nx == 1 || L.ny == 1 || L.nz == 1 || most > kRoundMax;
+    (wide ? k_bake_march<true> : k_bake_march<false>)<<<vox_grid(L), vox_block(), 0, s>>>(L, f.sigma_t, f.albedo,
+                                                                                         f.jsrc, m, accumulate);
     return cudaGetLastError();
 }
 
