@@ -77,7 +77,8 @@ bool same_params(const PassParams &a, const PassParams &b) {
            a.inv2h == b.inv2h && a.floor_ == b.floor_ && a.bf16 == b.bf16 && a.h2 == b.h2 && a.scheme == b.scheme &&
            a.tiled_f32 == b.tiled_f32 && a.tiled_fh == b.tiled_fh && a.quad_f32 == b.quad_f32 &&
            a.quad_fh == b.quad_fh && a.run_f32 == b.run_f32 && a.run_fh == b.run_fh &&
-           a.rows_f32 == b.rows_f32 && a.rows_fh == b.rows_fh && a.rows_ff == b.rows_ff && a.ff_form == b.ff_form;
+           a.rows_f32 == b.rows_f32 && a.rows_fh == b.rows_fh && a.rows_ff == b.rows_ff && a.ff_form == b.ff_form && a.direct == b.direct &&
+           a.early_f32 == b.early_f32 && a.early_fh == b.early_fh && a.early_ff == b.early_ff;
 }
 
 }  // namespace
@@ -362,9 +363,11 @@ fld_status ensure_alt(fld_grid_s *g) {
 
 // Whole iterations per launch pay where the launch and one memory latency are
 // most of a colour pass (measured, us per iteration against two launched passes:
-// 24^3 2.6 / 4.3, 32^3 2.7 / 4.2, hi/lo 3.3 / 4.2; 40^3 hi/lo 5.0 / 6.8; 50^3 5.3 /
-// 5.5; 64^3 8.5 / 6.1): above this size they are not tried.
+// 24^3 2.6 / 4.3, 32^3 2.7 / 4.2, hi/lo 3.3 / 4.1; 40^3 4.2 / 4.3, hi/lo 5.0 / 5.1; 50^3
+// 5.2 / 5.3; 64^3 8.5 / 5.2): above this size they are not tried.
 constexpr long long kRowsMaxVoxels = 250000;
+// Up to here the tuner also times passes that are not launched early (pass_early).
+constexpr long long kLateMaxVoxels = 600000;
 int rows_slot(Family fam) { return fam == FAM_F32 ? 0 : fam == FAM_FH ? 1 : 2; }
 
 // Tile of the whole-iteration launches of family fam; *ok: the grid can run them.
@@ -657,6 +660,7 @@ struct TuneChoice {
     int tiled = -1;           // blocked configuration id; launched passes: two unknowns per thread in tiles -1 or by
                               // running number -3, four per thread -2 (float-float: two with seven -1 or five
                               // -3 CTAs per SM, one -2); whole iterations -4
+    int early = 1;            // launched passes: early (programmatic dependent launch)
     int check_every = 64;
     double us_launched = 0.0, us_best = 0.0, us_check = 0.0;   // measured per iteration / per check
 };
@@ -680,7 +684,7 @@ std::string tune_path() {
 
 std::string tune_key(const fld_grid_s *g, Family fam, const PassParams &pp) {
     char b[192];
-    snprintf(b, sizeof(b), "v3 %dx%dx%d fam%d lim%d r%d bf%d sm%d", g->nx, g->ny, g->nz, (int)fam, pp.lim,
+    snprintf(b, sizeof(b), "v5 %dx%dx%d fam%d lim%d r%d bf%d sm%d", g->nx, g->ny, g->nz, (int)fam, pp.lim,
              pp.local_iters, pp.bf16, g->nsm);
     return b;
 }
@@ -699,7 +703,8 @@ void tune_load_locked() {
         std::string key = line;
         while (!key.empty() && key.back() == ' ') key.pop_back();
         TuneChoice c;
-        if (sscanf(bar + 1, "%d %d %lf %lf %lf", &c.tiled, &c.check_every, &c.us_launched, &c.us_best, &c.us_check) == 5 &&
+        if (sscanf(bar + 1, "%d %d %d %lf %lf %lf", &c.tiled, &c.early, &c.check_every, &c.us_launched, &c.us_best,
+                   &c.us_check) == 6 &&
             c.tiled >= -4 && c.tiled < kTiledConfigs && c.check_every >= 1)
             g_tune[key] = c;
     }
@@ -711,8 +716,8 @@ void tune_store_locked(const std::string &key, const TuneChoice &c) {
     const std::string path = tune_path();
     FILE *fp = path.empty() ? nullptr : fopen(path.c_str(), "a");
     if (!fp) return;
-    fprintf(fp, "%s | %d %d %.4f %.4f %.4f\n", key.c_str(), c.tiled, c.check_every, c.us_launched, c.us_best,
-            c.us_check);
+    fprintf(fp, "%s | %d %d %d %.4f %.4f %.4f\n", key.c_str(), c.tiled, c.early, c.check_every, c.us_launched,
+            c.us_best, c.us_check);
     fclose(fp);
 }
 
@@ -738,38 +743,60 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
     const int n = 16;   // iterations per timing, a multiple of every depth
     TuneChoice c;
     double best = INFINITY;
-    for (int cand = -4; cand < ncfg; ++cand) {
+    // (launches that are not early lose on all but small grids: not tried there)
+    const bool late = nvox(g) <= kLateMaxVoxels;
+    for (int ci = -8; ci < ncfg; ++ci) {
+        const int cand = ci < -4 ? ci + 4 : ci, early = ci < -4 ? 0 : 1;
+        if (!early && (!late || cand == -4)) continue;
         if (cand == -4 && !rows) continue;
         double t = INFINITY;
         PassParams pc = pp;
         pc.quad_f32 = pc.quad_fh = cand == -2 ? 1 : 0;
         pc.run_f32 = pc.run_fh = cand == -3 ? 1 : 0;
         pc.ff_form = cand == -2 ? 2 : cand == -3 ? 1 : 0;
-        for (int rep = 0; rep < 3; ++rep) {   // the first is a warm-up
-            FLD_CK(cudaEventRecord(g->evb0, g->stream));
+        pc.early_f32 = pc.early_fh = pc.early_ff = early;
+        // timed as a solve runs it, from a graph: launched one by one, small
+        // grids would show the host's pace
+        auto iterate = [&]() -> cudaError_t {
+            cudaError_t e = cudaSuccess;
             if (cand == -4) {
                 const float *const a[3] = {g->f.phi, g->f.D, g->f.phlo};
                 float *const b[3] = {g->alt_phi, g->alt_D, g->alt_lo};
-                for (int it = 0; it < n; ++it)
-                    FLD_CK(launch_rows(fam, g->L, g->f, pc, g->rtile[rows_slot(fam)], a, b, it == 0, g->stream));
+                for (int it = 0; it < n && e == cudaSuccess; ++it)
+                    e = launch_rows(fam, g->L, g->f, pc, g->rtile[rows_slot(fam)], a, b, it == 0, g->stream);
             } else if (cand < 0) {
-                for (int it = 0; it < n; ++it)
-                    for (int colour = 0; colour < 2; ++colour) FLD_CK(launch_pass(fam, g->L, fa, pc, colour, g->stream));
+                for (int it = 0; it < 2 * n && e == cudaSuccess; ++it)
+                    e = launch_pass(fam, g->L, fa, pc, it & 1, g->stream);
             } else {
-                for (int i = 0; i < n / tiled_depth(cand); ++i)
-                    FLD_CK(launch_tiled(fam, cand, g->L, g->f, pp, g->maps[cand][0], g->alt_phi, g->alt_D, g->alt_lo,
-                                        g->tiled_status, g->nsm, g->stream));
+                for (int i = 0; i < n / tiled_depth(cand) && e == cudaSuccess; ++i)
+                    e = launch_tiled(fam, cand, g->L, g->f, pp, g->maps[cand][0], g->alt_phi, g->alt_D, g->alt_lo,
+                                     g->tiled_status, g->nsm, g->stream);
             }
-            FLD_CK(cudaEventRecord(g->evb1, g->stream));
-            FLD_CK(cudaEventSynchronize(g->evb1));
+            return e;
+        };
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        FLD_CK(cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal));
+        const cudaError_t e1 = iterate(), e2 = cudaStreamEndCapture(g->stream, &graph);
+        cudaError_t ce = e1 != cudaSuccess ? e1 : e2;
+        if (ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        for (int rep = 0; rep < 3 && ce == cudaSuccess; ++rep) {   // the first is a warm-up
             float ms = 0.0f;
-            FLD_CK(cudaEventElapsedTime(&ms, g->evb0, g->evb1));
+            ce = cudaEventRecord(g->evb0, g->stream);
+            if (ce == cudaSuccess) ce = cudaGraphLaunch(exec, g->stream);
+            if (ce == cudaSuccess) ce = cudaEventRecord(g->evb1, g->stream);
+            if (ce == cudaSuccess) ce = cudaEventSynchronize(g->evb1);
+            if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, g->evb0, g->evb1);
             if (rep > 0) t = std::min(t, 1e3 * ms / n);
         }
-        if (cand == -1) c.us_launched = t;
+        if (exec) cudaGraphExecDestroy(exec);
+        if (ce != cudaSuccess) return cuda_fail(ce, "timing a sweep");
+        if (cand == -1 && early) c.us_launched = t;
         if (t < best) {
             best = t;
             c.tiled = cand;
+            c.early = early;
         }
     }
     if (ncfg > 0) g->tiled_used = true;   // surface a timeout of the timed blocked launches at the next check
@@ -801,6 +828,7 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
     pp->run_f32 = pp->run_fh = -1;
     pp->rows_f32 = pp->rows_fh = pp->rows_ff = 0;
     pp->ff_form = -1;
+    pp->early_f32 = pp->early_fh = pp->early_ff = -1;
     *ce = p->check_every > 0 ? p->check_every : 64;
     if (p->scheme != FLD_SCHEME_RED_BLACK || p->precision == FLD_PREC_FP64) return FLD_OK;
     fld_status st = FLD_OK;
@@ -850,12 +878,15 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
                 pp->tiled_f32 = shape;
                 pp->quad_f32 = quad;
                 pp->run_f32 = run;
+                pp->early_f32 = c.early;
             } else if (fam == FAM_FH) {
                 pp->tiled_fh = shape;
                 pp->quad_fh = quad;
                 pp->run_fh = run;
+                pp->early_fh = c.early;
             } else {
                 pp->ff_form = c.tiled == -2 ? 2 : c.tiled == -3 ? 1 : c.tiled == -1 ? 0 : -1;
+                pp->early_ff = c.early;
             }
         }
         if (k == 0 && p->check_every <= 0) *ce = c.check_every;
@@ -1556,6 +1587,7 @@ fld_status fld_iterate(fld_grid g, const fld_solve_params *p, int iterations) {
     PassParams pp = pass_params(g, p);
     int ce = 0;
     if ((st = choose_sweeps(g, p, &pp, &ce)) != FLD_OK) return st;
+    pp.direct = 1;
     return enqueue_iterations(g, fam, pp, iterations);
 }
 
@@ -2289,6 +2321,11 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
         for (size_t i = 0; i < nside; ++i) FLD_CK(cudaStreamWaitEvent(s->side[i], s->fork, 0));
         std::vector<int> k(n);
         std::vector<char> mixing(n, 0);
+        // whole-iteration launches repeat some updates to save launches: with
+        // enough other grids to fill the GPU the passes get more done
+        long long voxels = 0;
+        for (const ServerEntry &e : s->active) voxels += nvox(e.g);
+        const bool crowded = voxels > kRowsMaxVoxels;
         for (size_t i = 0; i < n; ++i) {
             const ServerEntry &e = s->active[i];
             k[i] = block_len(e.res.iterations, check_len(e.fam, p->precision, e.ce), p->max_iters, e.warm);
@@ -2369,7 +2406,12 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
                 e.acount = 0;
             }
             if (slot_of[i] < 0) {
-                st = run_block(e.g, e.fam, block_params(e.pp, e.res.iterations, e.warm), k[i]);
+                PassParams q = block_params(e.pp, e.res.iterations, e.warm);
+                if (crowded) q.rows_f32 = q.rows_fh = q.rows_ff = 0;   // (and early as without them)
+                if (crowded && e.pp.rows_f32) q.early_f32 = -1;
+                if (crowded && e.pp.rows_fh) q.early_fh = -1;
+                if (crowded && e.pp.rows_ff) q.early_ff = -1;
+                st = run_block(e.g, e.fam, q, k[i]);
                 s->launches += 2LL * k[i];
             } else {
                 std::vector<SweepDesc> &tab = tables[(size_t)slot_of[i]];

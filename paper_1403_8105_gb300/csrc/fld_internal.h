@@ -35,6 +35,10 @@ struct PassParams {
     // launched float-float passes: two unknowns per thread with seven (0) or five
     // (1) CTAs per SM, one unknown (2), or two by the size of the grid (-1)
     int ff_form = -1;
+    // passes launched early (programmatic dependent launch): 1, 0, or by the
+    // number of CTAs (-1); direct: launched one by one, not from a graph
+    int early_f32 = -1, early_fh = -1, early_ff = -1;
+    int direct = 0;
     // whole iterations per launch (fld_rows.cu)
     int rows_f32 = 0, rows_fh = 0, rows_ff = 0;
 };

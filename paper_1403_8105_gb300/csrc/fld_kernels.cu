@@ -830,16 +830,32 @@ __device__ __forceinline__ BatchDesc load_desc(const BatchDesc *__restrict__ p) 
     return d;
 }
 
-__global__ void __launch_bounds__(256) k_pass_d(Layout L, const double *__restrict__ sp,
+// FP64 colour pass.  The FP64 pipe takes 16 clocks a warp instruction (a 64th of
+// the FP32 rate) whatever its active lanes, so what counts is instructions times
+// warps.  Unknowns go by running number: a 32^3 grid's rows have 16 of a colour, and
+// tiles of 32 left half of every warp idle.  And quotients are combined:
+// R = g / d and 1 / R from one reciprocal of g d; Levermore-Pomraning as P / Q,
+// P = ((1 - r)(1 - e) + 2 e) r / sigma', Q = 1 - e, r = 1/R, e = exp(-2 R), so that D = P / Q and
+// delta = (P A / 2 + base Q) / ((sigma_a' h^2 + C / 2) Q + 3 P) share the reciprocal of Q times
+// that denominator.  Two reciprocals per round instead of six quotients, a few ulp.
+// 32^3: 19 -> 9.9 us a pass.
+constexpr int kPassDThreads = 64;
+
+template <int LIM, int ROUNDS>
+__global__ void __launch_bounds__(kPassDThreads) k_pass_d(Layout L, PassIndex ix, const double *__restrict__ sp,
                                                 const double *__restrict__ ah2, const double *__restrict__ jh2,
                                                 double *__restrict__ phi, double *__restrict__ D, int colour,
-                                                int lim, double larsen_n, double omega, double inv2h,
-                                                double floor_, int local_iters) {
+                                                int lim_rt, double larsen_n, double omega, double inv2h,
+                                                double floor_, int rounds_rt) {
+    pdl_launch_dependents();
+    const uint32_t e = blockIdx.x * (uint32_t)kPassDThreads + threadIdx.x;
+    if (e >= ix.total) return;
+    const uint32_t row = ix.by_items.quot(e);
+    const int K = (int)ix.by_rows.quot(row), J = (int)row - K * L.ny;
     Nbrs o;
-    if (!pass_cell(L, colour, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y + 1,
-                   blockIdx.z + 1, o) ||
-        blockIdx.y * blockDim.y + threadIdx.y >= L.ny)
-        return;
+    if (!pass_cell(L, colour, (int)(e - row * ix.per_row), J + 1, K + 1, o)) return;
+    const double s_ = sp[o.own], ah = ah2[o.own], jj = jh2[o.own];
+    pdl_wait();
     const double p0 = phi[o.own];
     double ps[6], Ds[6];
 #pragma unroll
@@ -847,8 +863,8 @@ __global__ void __launch_bounds__(256) k_pass_d(Layout L, const double *__restri
         ps[s] = phi[o.nb[s]];
         Ds[s] = D[o.nb[s]];
     }
-    const double s_ = sp[o.own], ah = ah2[o.own], jj = jh2[o.own];
     const double gx = ps[1] - ps[0], gy = ps[3] - ps[2], gz = ps[5] - ps[4];
+    const double gmax = fmax(inv2h * sqrt(fma(gx, gx, fma(gy, gy, gz * gz))), floor_);
     double A = 0.0, B = 0.0, C = 0.0;
 #pragma unroll
     for (int s = 0; s < 6; ++s) {
@@ -857,13 +873,39 @@ __global__ void __launch_bounds__(256) k_pass_d(Layout L, const double *__restri
         B = fma(Ds[s], d, B);
         C += Ds[s];
     }
-    const double base = fma(0.5, B, fma(-ah, p0, jj));
+    const double base = fma(0.5, B, fma(-ah, p0, jj)), den0 = fma(0.5, C, ah);
+    const double inv_sp = 1.0 / s_;
+    const int lim = LIM >= 0 ? LIM : lim_rt;
+    const int local_iters = ROUNDS > 0 ? ROUNDS : rounds_rt;
     double delta = 0.0, Dp = 0.0;
-    for (int r = 0; r < local_iters; ++r) {
-        Dp = knudsen_D_d(gx, gy, gz, inv2h, s_, p0 + delta, floor_, lim, larsen_n);
-        const double S = fma(0.5 * Dp, A, base);
-        const double den = (ah + 3.0 * Dp) + 0.5 * C;
-        delta = S / den;
+#pragma unroll(ROUNDS > 0 ? ROUNDS : 1)
+    for (int r = 0; r < (ROUNDS > 0 ? ROUNDS : local_iters); ++r) {
+        const double den = fmax(s_ * (p0 + delta), floor_);
+        double P, Q = 1.0;
+        // (the product of the two must stay a normal number)
+        const bool ranged = LIM == LIM_LP && gmax > 1e-130 && gmax < 1e130 && den > 1e-130 && den < 1e130;
+        if (ranged) {
+            const double both = 1.0 / (gmax * den);
+            const double R = gmax * gmax * both;
+            if (R < 0.2) {
+                P = lp_series_d(R) * inv_sp;
+            } else {
+                const double q = den * den * both;            // 1 / R
+                double w = 1.0 - q;
+                if (R < 20.0) {                                // exp(-40) is far below an ulp of 1 - 1/R
+                    const double ex = exp(-2.0 * R);
+                    Q = 1.0 - ex;
+                    w = fma(w, Q, 2.0 * ex);
+                }
+                P = w * q * inv_sp;
+            }
+        } else {
+            P = limiter_d(lim, larsen_n, gmax / den) * inv_sp;
+        }
+        const double N = fma(0.5 * P, A, base * Q), W = fma(3.0, P, den0 * Q);
+        const double both = 1.0 / (Q * W);
+        delta = N * Q * both;
+        Dp = P * W * both;
     }
     phi[o.own] = fma(omega, delta, p0);
     D[o.own] = Dp;
@@ -1457,10 +1499,10 @@ cudaError_t launch_d_to_f(const Layout &L, const double *src, float *hi, float *
     return cudaGetLastError();
 }
 
-// Launch with programmatic stream serialisation: the kernel may be scheduled
-// while the preceding grid in the stream finishes (see pdl_wait).
+// Launch with programmatic stream serialisation (early): the kernel may be
+// scheduled while the preceding grid in the stream finishes (see pdl_wait).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grd, dim3 blk, cudaStream_t s, Args... args) {
+cudaError_t launch_pdl(bool early, void (*k)(KArgs...), dim3 grd, dim3 blk, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grd;
     cfg.blockDim = blk;
@@ -1470,8 +1512,24 @@ cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grd, dim3 blk, cudaStream_t s, 
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+// Whether a pass of so many CTAs is launched early: as asked, or (-1) if it has
+// more than six per SM.  The CTAs of smaller ones, placed around those that still
+// run, end up two or three on some SMs and none on others, which can cost more
+// than the launch gap (us per iteration, early and not, FP32, hi/lo,
+// float-float: 50^3, 254 CTAs, 5.9 / 5.2, 7.2 / 5.6, 10.6 / 8.4, but 4.8 / 5.4 in FP32 on
+// a state further from the fixed point: the autotuner times both; 64^3, 512, 6.0 / 5.2, 6.1 /
+// 5.7, 8.5 / 7.9; 80^3, 1000, 6.6 / 6.5, 7.1 / 7.4, 11.0 / 11.5; 96^3, 1728, 7.7 / 8.8, 9.1 / 10.3,
+// 15.7 / 16.7; FP64 32^3, 256, 20 / 10).  Launches that do not come from a graph are
+// 4 us apart otherwise, and always early (FP64 passes take longer than that).
+constexpr long long kEarlyCtas = 912;
+inline bool pass_early(const PassParams &p, Family fam, dim3 g) {
+    const int asked = fam == FAM_F32 ? p.early_f32 : fam == FAM_FH ? p.early_fh : fam == FAM_FF ? p.early_ff : -1;
+    if (fam != FAM_F64 && p.direct) return true;
+    return asked >= 0 ? asked != 0 : (long long)g.x * g.y * g.z > kEarlyCtas;
 }
 
 cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const PassParams &p, int colour,
@@ -1489,7 +1547,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
                 constexpr bool B = decltype(bf)::value, H = decltype(hl)::value;
                 auto k = k_pass4<-1, 0, B, H>;
                 if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass4<LIM_LP, 2, B, H>;
-                return launch_pdl(k, grd4, blk4, s, L, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
+                return launch_pdl(pass_early(p, fam, grd4), k, grd4, blk4, s, L, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
                                   f.D, colour, p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h,
                                   (float)p.floor_, p.local_iters);
             };
@@ -1507,7 +1565,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
             else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_f32<LIM_LARSEN, 2, B, R>;
             PassIndex ix;
             const dim3 g2 = item_grid(L, pairs, R, &ix);
-            return launch_pdl(k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.D, colour,
+            return launch_pdl(pass_early(p, fam, g2), k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.D, colour,
                               p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_,
                               p.local_iters);
         };
@@ -1526,7 +1584,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
             if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass_ff<LIM_LP, 2>;
             else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass_ff<LIM_KERSHAW, 2>;
             else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass_ff<LIM_LARSEN, 2>;
-            return launch_pdl(k, grd, blk, s, L, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour, p.lim,
+            return launch_pdl(pass_early(p, fam, grd), k, grd, blk, s, L, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour, p.lim,
                               (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_, p.local_iters);
         }
         auto pick = [&](auto run) {
@@ -1538,7 +1596,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
                         ? k_pass2_ff<LIM_LP, 2, R, 5> : k_pass2_ff<LIM_LP, 2, R, 7>;
             else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass2_ff<LIM_KERSHAW, 2, R, 7>;
             else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_ff<LIM_LARSEN, 2, R, 7>;
-            return launch_pdl(k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour,
+            return launch_pdl(pass_early(p, fam, g2), k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour,
                               p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_,
                               p.local_iters);
         };
@@ -1553,7 +1611,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
             else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_fh<LIM_LARSEN, 2, B, R>;
             PassIndex ix;
             const dim3 g2 = item_grid(L, pairs, R, &ix);
-            return launch_pdl(k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
+            return launch_pdl(pass_early(p, fam, g2), k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
                               f.D, colour, p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h,
                               (float)p.floor_, p.local_iters);
         };
@@ -1562,9 +1620,16 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
         return p.bf16 ? pick(std::true_type{}, std::false_type{}) : pick(std::false_type{}, std::false_type{});
     }
     case FAM_F64:
-        k_pass_d<<<grd, blk, 0, s>>>(L, f.sp64, f.ah264, f.jh264, f.phi64, f.D64, colour, p.lim, p.larsen_n,
-                                    p.omega, p.inv2h, p.floor_, p.local_iters);
-        break;
+        {
+        PassIndex ix;
+        item_grid(L, (L.nx + 1) / 2, true, &ix);
+        auto k = k_pass_d<-1, 0>;
+        if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass_d<LIM_LP, 2>;
+        const dim3 gd((ix.total + kPassDThreads - 1) / kPassDThreads);
+        return launch_pdl(pass_early(p, fam, gd), k, gd, dim3(kPassDThreads), s, L, ix,
+                          f.sp64, f.ah264, f.jh264, f.phi64, f.D64, colour, p.lim, p.larsen_n, p.omega, p.inv2h,
+                          p.floor_, p.local_iters);
+        }
     }
     return cudaGetLastError();
 }
@@ -1614,7 +1679,7 @@ cudaError_t launch_pass_multi(const SweepDesc *descs, const int *counts, int hl,
     if (nctas <= 0) return cudaSuccess;
     auto k = hl ? (bf16 ? multi_kernel<true, true>(lim, local_iters) : multi_kernel<false, true>(lim, local_iters))
                 : (bf16 ? multi_kernel<true, false>(lim, local_iters) : multi_kernel<false, false>(lim, local_iters));
-    return launch_pdl(k, dim3(nctas), dim3(kMultiThreadsX, kMultiThreadsY, 1), s, descs, counts, colour);
+    return launch_pdl(true, k, dim3(nctas), dim3(kMultiThreadsX, kMultiThreadsY, 1), s, descs, counts, colour);
 }
 
 int reduction_blocks(const Layout &L) {

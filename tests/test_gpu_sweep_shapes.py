@@ -68,7 +68,7 @@ def test_whole_iteration_launches_equal_the_passes(tmp_path):
     import sys
 
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    lines = ["v3 %dx%dx%d fam%d lim%d r2 bf%d sm%d | -4 64 0 0 0" % (s[2], s[1], s[0], fam, lim, bf, sms)
+    lines = ["v5 %dx%dx%d fam%d lim%d r2 bf%d sm%d | -4 1 64 0 0 0" % (s[2], s[1], s[0], fam, lim, bf, sms)
              for s in ROWS_SHAPES for fam in (0, 1, 3) for lim in (fld.LIMITERS["lp"], fld.LIMITERS["larsen"])
              for bf in (0, 1)]
     cache = tmp_path / "tune.txt"
