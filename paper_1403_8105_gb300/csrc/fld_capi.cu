@@ -2006,6 +2006,8 @@ struct fld_server_s {
     BatchDesc *d_desc = nullptr;
     int *d_res = nullptr, *d_count = nullptr;
     double *d_part = nullptr, *d_out = nullptr;
+    double *d_dots = nullptr;           // Anderson dot products of cap_dots grids
+    int cap_dots = 0;
     int cap_grids = 0, cap_res = 0;
     std::vector<cudaStream_t> side;
     std::vector<cudaEvent_t> join;
@@ -2050,6 +2052,22 @@ fld_status server_workspace(fld_server_s *s, int grids, int res) {
     return FLD_OK;
 }
 
+// Room for the Anderson dot products of `grids` grids.
+fld_status server_dots(fld_server_s *s, int grids) {
+    if (s->p.anderson <= 0 || grids <= s->cap_dots) return FLD_OK;
+    FLD_CK(cudaStreamSynchronize(s->bs));
+    if (s->d_dots) cudaFree(s->d_dots);
+    s->d_dots = nullptr;
+    s->cap_dots = 0;
+    const int cap = grids + grids / 2 + 4;
+    if (cudaMalloc((void **)&s->d_dots, sizeof(double) * kAndersonMax * (size_t)cap) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return fail(FLD_ERR_OOM, "cudaMalloc of the dot products failed");
+    }
+    s->cap_dots = cap;
+    return FLD_OK;
+}
+
 double rel_from_sums(const fld_grid_s *g, int margin, double r2, double j2) {
     return rel_residual_from_sums(g->nx, g->ny, g->nz, g->h, margin, r2, j2);
 }
@@ -2066,6 +2084,24 @@ void server_retire(fld_server_s *s, size_t i, fld_status st, double rel) {
     e.g->stream = e.own_stream;
     s->done.push_back(e);
     s->active.erase(s->active.begin() + (long)i);
+}
+
+// A grid's work on another of the server's streams for a while.
+struct OnStream {
+    fld_grid_s *g;
+    cudaStream_t back;
+    OnStream(fld_grid_s *grid, cudaStream_t s) : g(grid), back(grid->stream) { g->stream = s; }
+    ~OnStream() { g->stream = back; }
+};
+
+// The server's stream waits for what its side streams hold.
+cudaError_t server_join(fld_server_s *s, size_t nside) {
+    for (size_t i = 0; i < nside; ++i) {
+        cudaError_t e = cudaEventRecord(s->join[i], s->side[i]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s->bs, s->join[i], 0);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // The device tables of the multi-grid launches (allocated on first use).
@@ -2210,8 +2246,10 @@ void fld_server_destroy(fld_server s) {
     if (!s) return;
     cudaSetDevice(s->device);
     if (s->bs) cudaStreamSynchronize(s->bs);
+    for (auto x : s->side) cudaStreamSynchronize(x);
     for (ServerEntry &e : s->active) e.g->stream = e.own_stream;   // grids go back to their owners
     server_free_workspace(s);
+    if (s->d_dots) cudaFree(s->d_dots);
     for (auto &kv : s->multi_graphs) cudaGraphExecDestroy(kv.second);
     for (int i = 0; i < kFuseSlots; ++i) {
         if (s->d_sweep[i]) cudaFree(s->d_sweep[i]);
@@ -2432,10 +2470,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
             if ((st = server_multi_block(s, (int)gi, tables[gi], table_items[gi], groups[gi].first, share,
                                          s->side[gi % nside])) != FLD_OK)
                 return st;
-        for (size_t i = 0; i < nside; ++i) {
-            FLD_CK(cudaEventRecord(s->join[i], s->side[i]));
-            FLD_CK(cudaStreamWaitEvent(s->bs, s->join[i], 0));
-        }
+        FLD_CK(server_join(s, nside));
         // -- residuals of all active grids in one batched pass
         // (grids in their FP64 sweeps are checked one by one, as fld_solve does)
         std::vector<BatchDesc> hd(n);
@@ -2481,12 +2516,16 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
             if ((st = residual_now(e.g, FAM_F64, e.pp, p->residual_margin, &rel64[i])) != FLD_OK) return st;
             s->launches += 3;
         }
-        // -- each grid's own decisions (same as fld_solve)
+        // -- each grid's own decisions (same as fld_solve).  Everything so far has
+        // finished (the residuals were read), so the grids' snapshots, conversions,
+        // images and mixes go to the side streams and overlap; one after another
+        // on the server's stream they took a third of a step of 16 small grids
         std::vector<std::pair<size_t, std::pair<fld_status, double>>> retire;
         std::vector<char> mix_now(n, 0);
         for (size_t i = 0; i < n; ++i) {
             ServerEntry &e = s->active[i];
             fld_grid_s *g = e.g;
+            const OnStream side(g, s->side[i % nside]);
             double rel = e.fam == FAM_F64 ? rel64[i] : rel_from_sums(g, p->residual_margin, out[2 * i], out[2 * i + 1]);
             e.res.rel_residual = rel;
             ++e.res.checks;
@@ -2562,6 +2601,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
         // readback, then each grid's weights and mix (same kernels and order
         // as fld_solve, so a grid's iterates are those of its solo solve)
         std::vector<double> dots(n * kAndersonMax);
+        if ((st = server_dots(s, (int)n)) != FLD_OK) return st;
         bool any_mix = false;
         for (size_t i = 0; i < n; ++i) {
             if (!mix_now[i]) continue;
@@ -2571,13 +2611,18 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
             float *hi, *lo;
             double *p64;
             anderson_state(e.g, e.fam, &hi, &lo, &p64);
-            FLD_CK(launch_anderson_collect(e.g->anderson, e.g->L, hi, lo, p64, slot, w, e.g->nsm, s->bs));
-            FLD_CK(cudaMemcpyAsync(&dots[i * kAndersonMax], e.g->anderson.dots, sizeof(double) * w,
-                                   cudaMemcpyDeviceToHost, s->bs));
+            AndersonBuffers b = e.g->anderson;
+            b.dots = s->d_dots + i * kAndersonMax;         // (read back together)
+            FLD_CK(launch_anderson_collect(b, e.g->L, hi, lo, p64, slot, w, e.g->nsm, s->side[i % nside]));
             s->launches += 2;
             any_mix = true;
         }
-        if (any_mix) FLD_CK(cudaStreamSynchronize(s->bs));
+        FLD_CK(server_join(s, nside));
+        if (any_mix) {
+            FLD_CK(cudaMemcpyAsync(dots.data(), s->d_dots, sizeof(double) * n * kAndersonMax, cudaMemcpyDeviceToHost,
+                                   s->bs));
+            FLD_CK(cudaStreamSynchronize(s->bs));
+        }
         for (size_t i = 0; i < n; ++i) {
             if (!mix_now[i]) continue;
             ServerEntry &e = s->active[i];
@@ -2593,7 +2638,8 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
                 float *hi, *lo;
                 double *p64;
                 anderson_state(e.g, e.fam, &hi, &lo, &p64);
-                FLD_CK(launch_anderson_mix(e.g->anderson, e.g->L, slot, w, wts, hi, lo, p64, e.g->nsm, s->bs));
+                FLD_CK(launch_anderson_mix(e.g->anderson, e.g->L, slot, w, wts, hi, lo, p64, e.g->nsm,
+                                           s->side[i % nside]));
                 s->launches += 1;
                 if (w > 1) ++e.res.anderson_steps;
             } else {
@@ -2601,6 +2647,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
                 e.have_x = false;
             }
         }
+        if (any_mix) FLD_CK(server_join(s, nside));
         for (size_t r = retire.size(); r-- > 0;) {
             ServerEntry &e = s->active[retire[r].first];
             if (e.fam == FAM_F64 && (st = sync_family(e.g, FAM_FF)) != FLD_OK) return st;   // as fld_solve
