@@ -78,7 +78,7 @@ bool same_params(const PassParams &a, const PassParams &b) {
            a.tiled_f32 == b.tiled_f32 && a.tiled_fh == b.tiled_fh && a.quad_f32 == b.quad_f32 &&
            a.quad_fh == b.quad_fh && a.run_f32 == b.run_f32 && a.run_fh == b.run_fh &&
            a.rows_f32 == b.rows_f32 && a.rows_fh == b.rows_fh && a.rows_ff == b.rows_ff && a.ff_form == b.ff_form && a.direct == b.direct &&
-           a.early_f32 == b.early_f32 && a.early_fh == b.early_fh && a.early_ff == b.early_ff;
+           a.single_f32 == b.single_f32 && a.single_fh == b.single_fh && a.early_f32 == b.early_f32 && a.early_fh == b.early_fh && a.early_ff == b.early_ff;
 }
 
 }  // namespace
@@ -362,10 +362,11 @@ fld_status ensure_alt(fld_grid_s *g) {
 }
 
 // Whole iterations per launch pay where the launch and one memory latency are
-// most of a colour pass (measured, us per iteration against two launched passes:
-// 24^3 2.6 / 4.3, 32^3 2.7 / 4.2, hi/lo 3.3 / 4.1; 40^3 4.2 / 4.3, hi/lo 5.0 / 5.1; 50^3
-// 5.2 / 5.3; 64^3 8.5 / 5.2): above this size they are not tried.
-constexpr long long kRowsMaxVoxels = 250000;
+// most of a colour pass (us per iteration against the best passes: hi/lo 24^3 2.8 /
+// 3.5, 32^3 3.3 / 3.7; 40^3 5.0 / 3.7; FP32 32^3 2.7 / 2.7): above this size they are not tried.
+// Launched one by one (fld_iterate) they have half the launches, which set the
+// pace up to about 40^3 (32^3 FP32, 16 iterations: 79 against 97 us).
+constexpr long long kRowsMaxVoxels = 100000, kRowsDirectVoxels = 70000;
 // Up to here the tuner also times passes that are not launched early (pass_early).
 constexpr long long kLateMaxVoxels = 600000;
 int rows_slot(Family fam) { return fam == FAM_F32 ? 0 : fam == FAM_FH ? 1 : 2; }
@@ -574,8 +575,11 @@ fld_status enqueue_iterations(fld_grid_s *g, Family fam, const PassParams &pp, i
                                done == 0, g->stream));
         if (nk) *nk = done + 2LL * (iters - done);
     }
-    for (int it = done; it < iters; ++it)
-        for (int colour = 0; colour < 2; ++colour) FLD_CK(launch_pass(fam, g->L, g->f, pp, colour, g->stream));
+    PassParams q = pp;
+    for (int i = 2 * done; i < 2 * iters; ++i) {
+        q.settle = (i - 2 * done) % kSettleEvery == 0;
+        FLD_CK(launch_pass(fam, g->L, g->f, q, i & 1, g->stream));
+    }
     return FLD_OK;
 }
 
@@ -659,7 +663,8 @@ void set_valid(fld_grid_s *g, Family fam) {
 struct TuneChoice {
     int tiled = -1;           // blocked configuration id; launched passes: two unknowns per thread in tiles -1 or by
                               // running number -3, four per thread -2 (float-float: two with seven -1 or five
-                              // -3 CTAs per SM, one -2); whole iterations -4
+                              // -3 CTAs per SM, one -2); whole iterations -4; one unknown per
+                              // thread -5
     int early = 1;            // launched passes: early (programmatic dependent launch)
     int check_every = 64;
     double us_launched = 0.0, us_best = 0.0, us_check = 0.0;   // measured per iteration / per check
@@ -684,7 +689,7 @@ std::string tune_path() {
 
 std::string tune_key(const fld_grid_s *g, Family fam, const PassParams &pp) {
     char b[192];
-    snprintf(b, sizeof(b), "v5 %dx%dx%d fam%d lim%d r%d bf%d sm%d", g->nx, g->ny, g->nz, (int)fam, pp.lim,
+    snprintf(b, sizeof(b), "v6 %dx%dx%d fam%d lim%d r%d bf%d sm%d", g->nx, g->ny, g->nz, (int)fam, pp.lim,
              pp.local_iters, pp.bf16, g->nsm);
     return b;
 }
@@ -705,7 +710,7 @@ void tune_load_locked() {
         TuneChoice c;
         if (sscanf(bar + 1, "%d %d %d %lf %lf %lf", &c.tiled, &c.early, &c.check_every, &c.us_launched, &c.us_best,
                    &c.us_check) == 6 &&
-            c.tiled >= -4 && c.tiled < kTiledConfigs && c.check_every >= 1)
+            c.tiled >= -5 && c.tiled < kTiledConfigs && c.check_every >= 1)
             g_tune[key] = c;
     }
     fclose(fp);
@@ -745,16 +750,18 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
     double best = INFINITY;
     // (launches that are not early lose on all but small grids: not tried there)
     const bool late = nvox(g) <= kLateMaxVoxels;
-    for (int ci = -8; ci < ncfg; ++ci) {
-        const int cand = ci < -4 ? ci + 4 : ci, early = ci < -4 ? 0 : 1;
-        if (!early && (!late || cand == -4)) continue;
-        if (cand == -4 && !rows) continue;
+    for (int ci = -10; ci < ncfg; ++ci) {
+        const int cand = ci < -5 ? ci + 5 : ci, early = ci < -5 ? 0 : 1;
+        if ((!early || cand == -5) && !late) continue;
+        if (cand == -4 && (!rows || !early)) continue;
+        if (cand == -5 && fam == FAM_FF) continue;     // (its -2)
         double t = INFINITY;
         PassParams pc = pp;
         pc.quad_f32 = pc.quad_fh = cand == -2 ? 1 : 0;
         pc.run_f32 = pc.run_fh = cand == -3 ? 1 : 0;
         pc.ff_form = cand == -2 ? 2 : cand == -3 ? 1 : 0;
         pc.early_f32 = pc.early_fh = pc.early_ff = early;
+        pc.single_f32 = pc.single_fh = cand == -5 ? 1 : 0;
         // timed as a solve runs it, from a graph: launched one by one, small
         // grids would show the host's pace
         auto iterate = [&]() -> cudaError_t {
@@ -765,8 +772,10 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
                 for (int it = 0; it < n && e == cudaSuccess; ++it)
                     e = launch_rows(fam, g->L, g->f, pc, g->rtile[rows_slot(fam)], a, b, it == 0, g->stream);
             } else if (cand < 0) {
-                for (int it = 0; it < 2 * n && e == cudaSuccess; ++it)
+                for (int it = 0; it < 2 * n && e == cudaSuccess; ++it) {
+                    pc.settle = it % kSettleEvery == 0;
                     e = launch_pass(fam, g->L, fa, pc, it & 1, g->stream);
+                }
             } else {
                 for (int i = 0; i < n / tiled_depth(cand) && e == cudaSuccess; ++i)
                     e = launch_tiled(fam, cand, g->L, g->f, pp, g->maps[cand][0], g->alt_phi, g->alt_D, g->alt_lo,
@@ -829,6 +838,7 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
     pp->rows_f32 = pp->rows_fh = pp->rows_ff = 0;
     pp->ff_form = -1;
     pp->early_f32 = pp->early_fh = pp->early_ff = -1;
+    pp->single_f32 = pp->single_fh = 0;
     *ce = p->check_every > 0 ? p->check_every : 64;
     if (p->scheme != FLD_SCHEME_RED_BLACK || p->precision == FLD_PREC_FP64) return FLD_OK;
     fld_status st = FLD_OK;
@@ -879,11 +889,13 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
                 pp->quad_f32 = quad;
                 pp->run_f32 = run;
                 pp->early_f32 = c.early;
+                pp->single_f32 = c.tiled == -5 ? 1 : 0;
             } else if (fam == FAM_FH) {
                 pp->tiled_fh = shape;
                 pp->quad_fh = quad;
                 pp->run_fh = run;
                 pp->early_fh = c.early;
+                pp->single_fh = c.tiled == -5 ? 1 : 0;
             } else {
                 pp->ff_form = c.tiled == -2 ? 2 : c.tiled == -3 ? 1 : c.tiled == -1 ? 0 : -1;
                 pp->early_ff = c.early;
@@ -1588,6 +1600,11 @@ fld_status fld_iterate(fld_grid g, const fld_solve_params *p, int iterations) {
     int ce = 0;
     if ((st = choose_sweeps(g, p, &pp, &ce)) != FLD_OK) return st;
     pp.direct = 1;
+    if (p->temporal_depth == 0 && p->scheme == FLD_SCHEME_RED_BLACK && fam != FAM_F64 && nvox(g) <= kRowsDirectVoxels) {
+        bool ok = false;
+        if ((st = ensure_rows(g, fam, pp, &ok)) != FLD_OK) return st;
+        if (ok) (fam == FAM_F32 ? pp.rows_f32 : fam == FAM_FH ? pp.rows_fh : pp.rows_ff) = 1;
+    }
     return enqueue_iterations(g, fam, pp, iterations);
 }
 
@@ -1985,6 +2002,8 @@ namespace {
 // Multi-grid tables a server step can fill (groups of grids with equal block
 // lengths; a further group runs grid by grid).
 constexpr int kFuseSlots = 8;
+// Voxels of active grids above which they fill the GPU together.
+constexpr long long kCrowdVoxels = 250000;
 
 // The state the Anderson kernels read and write for family fam.
 void anderson_state(fld_grid_s *g, Family fam, float **hi, float **lo, double **p64) {
@@ -2363,7 +2382,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
         // enough other grids to fill the GPU the passes get more done
         long long voxels = 0;
         for (const ServerEntry &e : s->active) voxels += nvox(e.g);
-        const bool crowded = voxels > kRowsMaxVoxels;
+        const bool crowded = voxels > kCrowdVoxels;
         for (size_t i = 0; i < n; ++i) {
             const ServerEntry &e = s->active[i];
             k[i] = block_len(e.res.iterations, check_len(e.fam, p->precision, e.ce), p->max_iters, e.warm);

@@ -35,10 +35,13 @@ struct PassParams {
     // launched float-float passes: two unknowns per thread with seven (0) or five
     // (1) CTAs per SM, one unknown (2), or two by the size of the grid (-1)
     int ff_form = -1;
+    // launched FP32 / hi/lo passes: one unknown per thread
+    int single_f32 = 0, single_fh = 0;
     // passes launched early (programmatic dependent launch): 1, 0, or by the
     // number of CTAs (-1); direct: launched one by one, not from a graph
     int early_f32 = -1, early_fh = -1, early_ff = -1;
     int direct = 0;
+    int settle = 0;      // of this launch: not early on a small grid (pass_early)
     // whole iterations per launch (fld_rows.cu)
     int rows_f32 = 0, rows_fh = 0, rows_ff = 0;
 };
@@ -133,6 +136,8 @@ cudaError_t launch_pack_from_d(const Layout &L, const double *src, double *dst, 
 cudaError_t launch_f_to_d(const Layout &L, const float *hi, const float *lo, double *dst, cudaStream_t s);
 cudaError_t launch_d_to_f(const Layout &L, const double *src, float *hi, float *lo, cudaStream_t s);
 
+// Passes from one that settles the placement of CTAs to the next (pass_early).
+constexpr int kSettleEvery = 8;
 // One colour pass of Algorithm 1 (colour 0 = red: i+j+k even).
 cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const PassParams &p, int colour,
                         cudaStream_t s);

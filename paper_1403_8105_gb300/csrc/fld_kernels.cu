@@ -428,7 +428,7 @@ __device__ __forceinline__ void tile_f32(const Layout &L, const float *__restric
 // them per SM: 13.7 -> 13.4 us per iteration at 128^3, 113.9 -> 108.9 at 256^3
 // against 256 threads.
 template <int LIM, int ROUNDS, bool BF, bool RUN>
-__global__ void __launch_bounds__(kPassThreads, 8) k_pass2_f32(Layout L, PassIndex ix, const float *__restrict__ sp,
+__global__ void __launch_bounds__(kPassThreads, 10) k_pass2_f32(Layout L, PassIndex ix, const float *__restrict__ sp,
                                                    const float *__restrict__ ah2, const float *__restrict__ jh2,
                                                    const uint16_t *__restrict__ spb,
                                                    const uint16_t *__restrict__ sab, float h2,
@@ -464,10 +464,10 @@ __device__ __forceinline__ void tile_fh(const Layout &L, const float *__restrict
     gather_pair(D, q, Ds0, Ds1);
     const float2 p0 = ld2(phi, q.own), l0 = ld2(phlo, q.own);
     float h0, lo0, d0, h1, lo1, d1;
-    cell_fh<LIM, ROUNDS>(p0.x, l0.x, ps0, ls0, Ds0, s2.x, a2.x, j2.x, lim_rt, larsen_n, omega, inv2h, floor_,
+    cell_fh<LIM, ROUNDS, true>(p0.x, l0.x, ps0, ls0, Ds0, s2.x, a2.x, j2.x, lim_rt, larsen_n, omega, inv2h, floor_,
                          rounds_rt, h0, lo0, d0);
     if (q.second) {
-        cell_fh<LIM, ROUNDS>(p0.y, l0.y, ps1, ls1, Ds1, s2.y, a2.y, j2.y, lim_rt, larsen_n, omega, inv2h, floor_,
+        cell_fh<LIM, ROUNDS, true>(p0.y, l0.y, ps1, ls1, Ds1, s2.y, a2.y, j2.y, lim_rt, larsen_n, omega, inv2h, floor_,
                              rounds_rt, h1, lo1, d1);
         *reinterpret_cast<float2 *>(phi + q.own) = make_float2(h0, h1);
         *reinterpret_cast<float2 *>(phlo + q.own) = make_float2(lo0, lo1);
@@ -494,6 +494,43 @@ __global__ void __launch_bounds__(kPassThreads, 8) k_pass2_fh(Layout L, PassInde
     if (!pass_item<RUN>(L, ix, t, J, K)) return;
     tile_fh<LIM, ROUNDS, BF>(L, sp, ah2, jh2, spb, sab, h2, phi, phlo, D, colour, lim_rt, larsen_n, omega, inv2h,
                              floor_, rounds_rt, 2 * t, J, K);
+}
+
+// One unknown per thread, FP32 or hi/lo, the limiter without branches: on grids too
+// small to fill the GPU a pass takes as long as one thread's chain of dependent
+// operations, which the pair pass goes through twice (us per iteration, pairs and
+// this, timed by the tuner: 32^3 FP32 4.1 / 2.8, 50^3 4.5 / 3.5, hi/lo 5.4 / 4.8; 80^3 6.9 / 6.1).
+template <int LIM, int ROUNDS, bool HL>
+__global__ void __launch_bounds__(kPassThreads) k_pass1(Layout L, PassIndex ix, const float *__restrict__ sp,
+                                                        const float *__restrict__ ah2,
+                                                        const float *__restrict__ jh2, float *__restrict__ phi,
+                                                        float *__restrict__ phlo, float *__restrict__ D, int colour,
+                                                        int lim_rt, float larsen_n, float omega, float inv2h,
+                                                        float floor_, int rounds_rt) {
+    pdl_launch_dependents();
+    int t, J, K;
+    Nbrs o;
+    if (!pass_item<true>(L, ix, t, J, K) || !pass_cell(L, colour, t, J, K, o)) return;
+    const float s_ = sp[o.own], ah = ah2[o.own], jj = jh2[o.own];
+    pdl_wait();
+    const float p0 = phi[o.own], p0lo = HL ? phlo[o.own] : 0.0f;
+    float ps[6], ls[6], Ds[6];
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+        ps[s] = phi[o.nb[s]];
+        if (HL) ls[s] = phlo[o.nb[s]];
+        Ds[s] = D[o.nb[s]];
+    }
+    float hi, lo, Dp;
+    if (HL) {
+        cell_fh<LIM, ROUNDS, true>(p0, p0lo, ps, ls, Ds, s_, ah, jj, lim_rt, larsen_n, omega, inv2h, floor_,
+                                   rounds_rt, hi, lo, Dp);
+        phlo[o.own] = lo;
+    } else {
+        cell_f32<LIM, ROUNDS, true>(p0, ps, Ds, s_, ah, jj, lim_rt, larsen_n, omega, inv2h, floor_, rounds_rt, hi, Dp);
+    }
+    phi[o.own] = hi;
+    D[o.own] = Dp;
 }
 
 // Four adjacent unknowns t .. t+3 (t a multiple of 4) of one colour in row
@@ -838,7 +875,7 @@ __device__ __forceinline__ BatchDesc load_desc(const BatchDesc *__restrict__ p) 
 // P = ((1 - r)(1 - e) + 2 e) r / sigma', Q = 1 - e, r = 1/R, e = exp(-2 R), so that D = P / Q and
 // delta = (P A / 2 + base Q) / ((sigma_a' h^2 + C / 2) Q + 3 P) share the reciprocal of Q times
 // that denominator.  Two reciprocals per round instead of six quotients, a few ulp.
-// 32^3: 19 -> 9.9 us a pass.
+// 32^3: 19 -> 9.7 us a pass.
 constexpr int kPassDThreads = 64;
 
 template <int LIM, int ROUNDS>
@@ -1516,20 +1553,25 @@ cudaError_t launch_pdl(bool early, void (*k)(KArgs...), dim3 grd, dim3 blk, cuda
     return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
-// Whether a pass of so many CTAs is launched early: as asked, or (-1) if it has
-// more than six per SM.  The CTAs of smaller ones, placed around those that still
-// run, end up two or three on some SMs and none on others, which can cost more
-// than the launch gap (us per iteration, early and not, FP32, hi/lo,
-// float-float: 50^3, 254 CTAs, 5.9 / 5.2, 7.2 / 5.6, 10.6 / 8.4, but 4.8 / 5.4 in FP32 on
-// a state further from the fixed point: the autotuner times both; 64^3, 512, 6.0 / 5.2, 6.1 /
-// 5.7, 8.5 / 7.9; 80^3, 1000, 6.6 / 6.5, 7.1 / 7.4, 11.0 / 11.5; 96^3, 1728, 7.7 / 8.8, 9.1 / 10.3,
-// 15.7 / 16.7; FP64 32^3, 256, 20 / 10).  Launches that do not come from a graph are
-// 4 us apart otherwise, and always early (FP64 passes take longer than that).
-constexpr long long kEarlyCtas = 912;
-inline bool pass_early(const PassParams &p, Family fam, dim3 g) {
-    const int asked = fam == FAM_F32 ? p.early_f32 : fam == FAM_FH ? p.early_fh : fam == FAM_FF ? p.early_ff : -1;
+// Whether a pass of so many CTAs is launched early.  The CTAs of a small grid, placed
+// around those of the preceding pass that still run, end up two or three on some SMs and
+// none on others, and from pass to pass the placement gets worse (50^3 FP32, us per
+// iteration: 3.5 over 16 iterations, 4.1 over 64, 5.5 over 512; never early 4.3).  So every
+// kSettleEvery-th of their passes waits for the preceding one to end, and the
+// next start from an even placement again: 3.2.  Measured so, FP32 / hi/lo / float-float:
+// 32^3 2.7 / 3.3 / 4.5 (all early 2.6 / 3.3 / 5.2), 50^3 3.2 / 4.5 / 6.4 (5.5 / 7.2 / 6.6), 64^3 4.2 / 5.3 / 8.0
+// (6.1 / 5.4 / 8.0); 4, 16 and 32 launches differ by 3 %.  From 80^3 on all early is as fast
+// or faster (96^3 7.7 against 7.9).  Otherwise as asked by the tuner, or (-1) if there
+// are more than six CTAs per SM.  Launches that do not come from a graph are 4 us apart
+// unless early, which is worse than any placement; FP64 passes take longer than that
+// (32^3, a pass in a graph: all early 20 us, never 9.9, settled 9.7).
+constexpr long long kEarlyCtas = 912, kSettleCtas = 1216;
+bool pass_early(const PassParams &p, Family fam, dim3 g) {
+    const long long ctas = (long long)g.x * g.y * g.z;
     if (fam != FAM_F64 && p.direct) return true;
-    return asked >= 0 ? asked != 0 : (long long)g.x * g.y * g.z > kEarlyCtas;
+    if (p.settle && ctas <= kSettleCtas) return false;
+    const int asked = fam == FAM_F32 ? p.early_f32 : fam == FAM_FH ? p.early_fh : fam == FAM_FF ? p.early_ff : 1;
+    return asked >= 0 ? asked != 0 : ctas > kEarlyCtas;
 }
 
 cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const PassParams &p, int colour,
@@ -1537,6 +1579,15 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
     const dim3 blk(32, 8, 1);
     const dim3 grd = pass_grid(L, blk);
     const int pairs = ((L.nx + 1) / 2 + 1) / 2;
+    if (fam != FAM_F64 && fam != FAM_FF && (fam == FAM_F32 ? p.single_f32 : p.single_fh)) {
+        PassIndex ix;
+        const dim3 g1 = item_grid(L, (L.nx + 1) / 2, true, &ix);
+        auto k = fam == FAM_FH ? k_pass1<-1, 0, true> : k_pass1<-1, 0, false>;
+        if (p.local_iters == 2 && p.lim == LIM_LP) k = fam == FAM_FH ? k_pass1<LIM_LP, 2, true> : k_pass1<LIM_LP, 2, false>;
+        return launch_pdl(pass_early(p, fam, g1), k, g1, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.phi,
+                          f.phlo, f.D, colour, p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h,
+                          (float)p.floor_, p.local_iters);
+    }
     switch (fam) {
     case FAM_F32:
     case FAM_FH:
