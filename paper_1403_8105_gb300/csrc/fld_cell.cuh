@@ -277,15 +277,19 @@ struct FFTerms2 {
     float2 A, nA, nAlo, C;       // A.hi, and both words of A negated
 };
 
-// |grad phi|, floored (grad_floor_f of ff_terms' differences).
+// |grad phi|, floored (grad_floor_f of ff_terms' differences).  Without LO the low
+// words are zero, here and below.
+template <bool LO = true>
 __device__ __forceinline__ float2 grad_pair(const float2 ps[6], const float2 ls[6], float inv2h, float floor_) {
-    const float2 gx = mul2(add2(sub2(ps[1], ps[0]), sub2(ls[1], ls[0])), both(inv2h));
-    const float2 gy = mul2(add2(sub2(ps[3], ps[2]), sub2(ls[3], ls[2])), both(inv2h));
-    const float2 gz = mul2(add2(sub2(ps[5], ps[4]), sub2(ls[5], ls[4])), both(inv2h));
+    const float2 dx = sub2(ps[1], ps[0]), dy = sub2(ps[3], ps[2]), dz = sub2(ps[5], ps[4]);
+    const float2 gx = mul2(LO ? add2(dx, sub2(ls[1], ls[0])) : dx, both(inv2h));
+    const float2 gy = mul2(LO ? add2(dy, sub2(ls[3], ls[2])) : dy, both(inv2h));
+    const float2 gz = mul2(LO ? add2(dz, sub2(ls[5], ls[4])) : dz, both(inv2h));
     const float2 g2 = fma2(gx, gx, fma2(gy, gy, mul2(gz, gz)));
     return make_float2(fmaxf(sqrtf(g2.x), floor_), fmaxf(sqrtf(g2.y), floor_));
 }
 
+template <bool LO = true>
 __device__ __forceinline__ FFTerms2 ff_terms_pair(float2 p0, float2 p0lo, const float2 ps[6], const float2 ls[6],
                                                   const float2 Ds[6], float2 ah, float2 jj) {
     FFTerms2 T;
@@ -295,7 +299,7 @@ __device__ __forceinline__ FFTerms2 ff_terms_pair(float2 p0, float2 p0lo, const 
 #pragma unroll
     for (int s = 0; s < 6; ++s) {
         const ff2 dh = two_sum2(ps[s], np0);
-        const float2 dl = add2(sub2(ls[s], p0lo), dh.lo);
+        const float2 dl = LO ? add2(sub2(ls[s], p0lo), dh.lo) : dh.lo;
         const float2 nD = neg2(Ds[s]);
         const float2 p = mul2(Ds[s], dh.hi);
         const float2 npe = fma2(nD, dl, fma2(nD, dh.hi, p));
@@ -317,7 +321,8 @@ __device__ __forceinline__ FFTerms2 ff_terms_pair(float2 p0, float2 p0lo, const 
     const float2 nBlo = add2(nBl, sub2(B, Bh));
     // base = j h^2 - sigma_a' h^2 phi + B / 2
     const float2 P = mul2(p0, ah);
-    const float2 e = fma2(neg2(p0lo), ah, fma2(np0, ah, P));
+    const float2 pl = fma2(np0, ah, P);
+    const float2 e = LO ? fma2(neg2(p0lo), ah, pl) : pl;
     const float2 mh = sub2(e, P);
     const float2 ml = sub2(e, add2(mh, P));
     const ff2 t = two_sum2(mh, jj);

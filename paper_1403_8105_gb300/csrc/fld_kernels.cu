@@ -153,29 +153,44 @@ __global__ void k_prep_d(Layout L, const float *__restrict__ st, const float *__
 }
 
 // Every element of both colour arrays: unknowns get (phi0, D0), the ghost
-// layer (phi_b, D_b), the alignment slack of each half row 0.
+// layer (phi_b, D_b), the alignment slack of each half row 0.  Four elements of
+// a half row per thread, stored together (512^3: 552 -> 261 us).
 template <typename T>
-__global__ void k_init(Layout L, T *__restrict__ phi, float *__restrict__ phlo, T *__restrict__ D, T phi0, T D0,
-                       T phi_b, T D_b) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= L.total) return;
-    const int c = e >= L.cs ? 1 : 0;
-    const int r = e - c * L.cs;
-    const int K = r / (L.hpx * L.py);
-    const int w = r - K * (L.hpx * L.py);
-    const int J = w / L.hpx;
-    const int pos = w - J * L.hpx - kXoff;            // = (I + 1) >> 1 for a cell
-    const int par = (J + K + 1 + c) & 1;               // I & 1 of this row's cells
-    const int I = par ? 2 * pos - 1 : 2 * pos;
-    T p = T(0), d = T(0);
-    if (pos >= 0 && I >= 0 && I <= L.nx + 1) {
-        const bool ghost = I == 0 || J == 0 || K == 0 || I == L.nx + 1 || J == L.ny + 1 || K == L.nz + 1;
-        p = ghost ? phi_b : phi0;
-        d = ghost ? D_b : D0;
+__device__ __forceinline__ void store4(T *p, const T v[4]) {
+    if (sizeof(T) == 4) {
+        *reinterpret_cast<float4 *>(p) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+    } else {
+        reinterpret_cast<double2 *>(p)[0] = make_double2((double)v[0], (double)v[1]);
+        reinterpret_cast<double2 *>(p)[1] = make_double2((double)v[2], (double)v[3]);
     }
-    phi[e] = p;
-    D[e] = d;
-    if (phlo) phlo[e] = 0.0f;
+}
+
+template <typename T>
+__global__ void k_init(Layout L, Divisor by_quads, Divisor by_py, T *__restrict__ phi, float *__restrict__ phlo,
+                       T *__restrict__ D, T phi0, T D0, T phi_b, T D_b) {
+    const uint32_t e4 = blockIdx.x * blockDim.x + threadIdx.x;      // quad of elements
+    if (e4 >= (uint32_t)L.total >> 2) return;
+    const uint32_t row = by_quads.quot(e4);                         // row of either colour
+    const int rows = L.py * (L.nz + 2), c = (int)row >= rows ? 1 : 0;
+    const uint32_t r = row - c * rows;
+    const int K = (int)by_py.quot(r), J = (int)r - K * L.py;
+    const int par = (J + K + 1 + c) & 1;                            // I & 1 of this row's cells
+    T p[4], d[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int pos = 4 * (int)(e4 - row * ((uint32_t)L.hpx >> 2)) + u - kXoff;   // = (I + 1) >> 1 for a cell
+        const int I = par ? 2 * pos - 1 : 2 * pos;
+        p[u] = d[u] = T(0);
+        if (pos >= 0 && I >= 0 && I <= L.nx + 1) {
+            const bool ghost = I == 0 || J == 0 || K == 0 || I == L.nx + 1 || J == L.ny + 1 || K == L.nz + 1;
+            p[u] = ghost ? phi_b : phi0;
+            d[u] = ghost ? D_b : D0;
+        }
+    }
+    store4(phi + 4 * (size_t)e4, p);
+    store4(D + 4 * (size_t)e4, d);
+    const float zero[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (phlo) store4(phlo + 4 * (size_t)e4, zero);
 }
 
 // Packed (nx+2)(ny+2)(nz+2) <-> device layout.  A thread moves four values a
@@ -959,7 +974,7 @@ __global__ void __launch_bounds__(kPassDThreads) k_pass_d(Layout L, PassIndex ix
 // for the last block to add: at 256^3 fresh D, residual and final sum took 104,
 // 362 and 79 us.
 constexpr int kCheckThreads = 128;
-constexpr int kCheckCtas = 1824;       // twelve per SM of 152
+constexpr int kCheckCtas = 2128;       // two waves of the residual's seven per SM of 152
 
 template <typename F>
 __device__ __forceinline__ void for_pairs(const Layout &L, const CheckIndex &ix, int cta, int ctas, F &&body) {
@@ -986,11 +1001,8 @@ __device__ __forceinline__ void fresh_D_pairs(const Layout &L, const CheckIndex 
         float2 ps[6], ls[6];
         gather_packed(phi, q, ps);
         if (LO) gather_packed(phlo, q, ls);
-        else
-#pragma unroll
-            for (int s = 0; s < 6; ++s) ls[s] = both(0.0f);
         const float2 s2 = ld2(sp, q.own), p0 = ld2(phi, q.own);
-        const float2 g = grad_pair(ps, ls, inv2h, floor_);
+        const float2 g = grad_pair<LO>(ps, ls, inv2h, floor_);
         const float dx = D_of_f(D_point(g.x, s2.x), p0.x, floor_, lim, larsen_n);
         if (q.second) {
             const float dy = D_of_f(D_point(g.y, s2.y), p0.y, floor_, lim, larsen_n);
@@ -1039,9 +1051,6 @@ __device__ __forceinline__ void residual_pairs(const Layout &L, const CheckIndex
         float2 ps[6], ls[6], Ds[6];
         gather_packed(phi, q, ps);
         if (LO) gather_packed(phlo, q, ls);
-        else
-#pragma unroll
-            for (int s = 0; s < 6; ++s) ls[s] = both(0.0f);
         const int I0 = 2 * t + 2 - ((J + K + 1 + c) & 1);      // padded I of the first unknown
         // ghost neighbours keep their Dirichlet D (never recomputed)
         const float2 xv = ld2(Df, q.xv);
@@ -1055,7 +1064,7 @@ __device__ __forceinline__ void residual_pairs(const Layout &L, const CheckIndex
         Ds[4] = ld2(K == 1 ? Dghost : Df, q.zm);
         Ds[5] = ld2(K == L.nz ? Dghost : Df, q.zp);
         const float2 jj = ld2(jh2, q.own);
-        const FFTerms2 T = ff_terms_pair(ld2(phi, q.own), LO ? ld2(phlo, q.own) : both(0.0f), ps, ls, Ds,
+        const FFTerms2 T = ff_terms_pair<LO>(ld2(phi, q.own), LO ? ld2(phlo, q.own) : both(0.0f), ps, ls, Ds,
                                          ld2(ah2, q.own), jj);
         const ff2 S = ff_S_pair(T, ld2(Df, q.own));
         const ff sx{S.hi.x, S.lo.x}, sy{S.hi.y, S.lo.y};
@@ -1484,16 +1493,22 @@ cudaError_t launch_prep_d(const Layout &L, const Fields &f, double sigma_eps, do
 cudaError_t launch_init_f(const Layout &L, float *phi, float *phlo, float *D, double phi0, double D0, double phi_b,
                           double D_b, cudaStream_t s) {
     const int blk = 256;
-    const int nb = (L.total + blk - 1) / blk;
-    k_init<float><<<nb, blk, 0, s>>>(L, phi, phlo, D, (float)phi0, (float)D0, (float)phi_b, (float)D_b);
+    const int nb = (L.total / 4 + blk - 1) / blk;
+    Divisor by_quads, by_py;
+    by_quads.set((uint32_t)L.hpx / 4);
+    by_py.set((uint32_t)L.py);
+    k_init<float><<<nb, blk, 0, s>>>(L, by_quads, by_py, phi, phlo, D, (float)phi0, (float)D0, (float)phi_b, (float)D_b);
     return cudaGetLastError();
 }
 
 cudaError_t launch_init_d(const Layout &L, double *phi, double *D, double phi0, double D0, double phi_b, double D_b,
                           cudaStream_t s) {
     const int blk = 256;
-    const int nb = (L.total + blk - 1) / blk;
-    k_init<double><<<nb, blk, 0, s>>>(L, phi, nullptr, D, phi0, D0, phi_b, D_b);
+    const int nb = (L.total / 4 + blk - 1) / blk;
+    Divisor by_quads, by_py;
+    by_quads.set((uint32_t)L.hpx / 4);
+    by_py.set((uint32_t)L.py);
+    k_init<double><<<nb, blk, 0, s>>>(L, by_quads, by_py, phi, nullptr, D, phi0, D0, phi_b, D_b);
     return cudaGetLastError();
 }
 
