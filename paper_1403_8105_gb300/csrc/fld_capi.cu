@@ -77,7 +77,7 @@ bool same_params(const PassParams &a, const PassParams &b) {
            a.inv2h == b.inv2h && a.floor_ == b.floor_ && a.bf16 == b.bf16 && a.h2 == b.h2 && a.scheme == b.scheme &&
            a.tiled_f32 == b.tiled_f32 && a.tiled_fh == b.tiled_fh && a.quad_f32 == b.quad_f32 &&
            a.quad_fh == b.quad_fh && a.run_f32 == b.run_f32 && a.run_fh == b.run_fh &&
-           a.rows_f32 == b.rows_f32 && a.rows_fh == b.rows_fh && a.rows_ff == b.rows_ff && a.ff_form == b.ff_form && a.direct == b.direct &&
+           a.rows_f32 == b.rows_f32 && a.rows_fh == b.rows_fh && a.ff_form == b.ff_form && a.direct == b.direct &&
            a.single_f32 == b.single_f32 && a.single_fh == b.single_fh && a.early_f32 == b.early_f32 && a.early_fh == b.early_fh && a.early_ff == b.early_ff;
 }
 
@@ -118,7 +118,7 @@ struct fld_grid_s {
     AndersonBuffers anderson{};
     int anderson_slots = 0;
     int nsm = 0;
-    RowsTile rtile[3] = {{0, 0}, {0, 0}, {0, 0}};   // tiles of whole-iteration launches (rows_slot)
+    RowsTile rtile[2] = {{0, 0}, {0, 0}};   // tiles of whole-iteration launches (rows_slot)
     // temporally blocked sweeps: the other buffers of the ping-pong pair, the
     // kernels' timeout flag and the TMA descriptors (made on first use)
     float *alt_phi = nullptr, *alt_D = nullptr, *alt_lo = nullptr;
@@ -369,12 +369,12 @@ fld_status ensure_alt(fld_grid_s *g) {
 constexpr long long kRowsMaxVoxels = 100000, kRowsDirectVoxels = 70000;
 // Up to here the tuner also times passes that are not launched early (pass_early).
 constexpr long long kLateMaxVoxels = 600000;
-int rows_slot(Family fam) { return fam == FAM_F32 ? 0 : fam == FAM_FH ? 1 : 2; }
+int rows_slot(Family fam) { return fam == FAM_F32 ? 0 : 1; }
 
 // Tile of the whole-iteration launches of family fam; *ok: the grid can run them.
 fld_status ensure_rows(fld_grid_s *g, Family fam, const PassParams &pp, bool *ok) {
     *ok = false;
-    if (nvox(g) > kRowsMaxVoxels) return FLD_OK;
+    if (nvox(g) > kRowsMaxVoxels || (fam != FAM_F32 && fam != FAM_FH)) return FLD_OK;
     RowsTile &t = g->rtile[rows_slot(fam)];
     if (t.TJ == 0) t = rows_tile(g->L, fam, g->nsm);
     if (t.TJ == 0) return FLD_OK;
@@ -565,7 +565,7 @@ fld_status enqueue_iterations(fld_grid_s *g, Family fam, const PassParams &pp, i
             g->tiled_used = true;
         }
     }
-    if (fam == FAM_F32 ? pp.rows_f32 : fam == FAM_FH ? pp.rows_fh : fam == FAM_FF ? pp.rows_ff : 0) {
+    if (fam == FAM_F32 ? pp.rows_f32 : fam == FAM_FH ? pp.rows_fh : 0) {
         // whole iterations per launch, an even number of them (ping-pong); the
         // first also brings the ghosts to the second buffers
         if (!g->alt_phi) return fail(FLD_ERR_STATE, "whole-iteration sweeps were not prepared");
@@ -577,7 +577,7 @@ fld_status enqueue_iterations(fld_grid_s *g, Family fam, const PassParams &pp, i
     }
     PassParams q = pp;
     for (int i = 2 * done; i < 2 * iters; ++i) {
-        q.settle = (i - 2 * done) % kSettleEvery == 0;
+        q.settle = i == 0 ? 2 : (i - 2 * done) % kSettleEvery == 0;
         FLD_CK(launch_pass(fam, g->L, g->f, q, i & 1, g->stream));
     }
     return FLD_OK;
@@ -835,7 +835,7 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
     pp->tiled_f32 = pp->tiled_fh = -1;
     pp->quad_f32 = pp->quad_fh = p->cells_per_thread == 4 ? 1 : 0;
     pp->run_f32 = pp->run_fh = -1;
-    pp->rows_f32 = pp->rows_fh = pp->rows_ff = 0;
+    pp->rows_f32 = pp->rows_fh = 0;
     pp->ff_form = -1;
     pp->early_f32 = pp->early_fh = pp->early_ff = -1;
     pp->single_f32 = pp->single_fh = 0;
@@ -880,7 +880,7 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
             if (c.tiled == -4) {
                 bool ok = false;
                 if ((st = ensure_rows(g, fam, *pp, &ok)) != FLD_OK) return st;
-                (fam == FAM_F32 ? pp->rows_f32 : fam == FAM_FH ? pp->rows_fh : pp->rows_ff) = ok ? 1 : 0;
+                if (fam != FAM_FF) (fam == FAM_F32 ? pp->rows_f32 : pp->rows_fh) = ok ? 1 : 0;
             }
             const int shape = c.tiled >= 0 ? c.tiled : -1;
             const int quad = c.tiled == -2 ? 1 : 0, run = c.tiled == -3 ? 1 : c.tiled == -1 ? 0 : -1;
@@ -1600,10 +1600,10 @@ fld_status fld_iterate(fld_grid g, const fld_solve_params *p, int iterations) {
     int ce = 0;
     if ((st = choose_sweeps(g, p, &pp, &ce)) != FLD_OK) return st;
     pp.direct = 1;
-    if (p->temporal_depth == 0 && p->scheme == FLD_SCHEME_RED_BLACK && fam != FAM_F64 && nvox(g) <= kRowsDirectVoxels) {
+    if (p->temporal_depth == 0 && p->scheme == FLD_SCHEME_RED_BLACK && nvox(g) <= kRowsDirectVoxels) {
         bool ok = false;
         if ((st = ensure_rows(g, fam, pp, &ok)) != FLD_OK) return st;
-        if (ok) (fam == FAM_F32 ? pp.rows_f32 : fam == FAM_FH ? pp.rows_fh : pp.rows_ff) = 1;
+        if (ok) (fam == FAM_F32 ? pp.rows_f32 : pp.rows_fh) = 1;
     }
     return enqueue_iterations(g, fam, pp, iterations);
 }
@@ -2467,7 +2467,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
                 if (crowded) {
                     // (the pair passes, launched early throughout: 16 clouds of
                     // 32^3 to 64^3 104 -> 93 ms; whole iterations 129)
-                    q.rows_f32 = q.rows_fh = q.rows_ff = 0;
+                    q.rows_f32 = q.rows_fh = 0;
                     q.single_f32 = q.single_fh = 0;
                     q.run_f32 = q.run_fh = -1;
                     q.direct = 1;

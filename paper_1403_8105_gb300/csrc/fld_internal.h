@@ -41,9 +41,11 @@ struct PassParams {
     // number of CTAs (-1); direct: launched one by one, not from a graph
     int early_f32 = -1, early_fh = -1, early_ff = -1;
     int direct = 0;
-    int settle = 0;      // of this launch: not early on a small grid (pass_early)
+    // of this launch: not early on a small grid (1), or not at all (2: the first of
+    // a run, whose medium the kernels before it may have written)
+    int settle = 0;
     // whole iterations per launch (fld_rows.cu)
-    int rows_f32 = 0, rows_fh = 0, rows_ff = 0;
+    int rows_f32 = 0, rows_fh = 0;
 };
 
 // Device fields of one grid (padded layout unless noted).
@@ -271,15 +273,15 @@ cudaError_t launch_tiled(Family fam, int id, const Layout &L, const Fields &f, c
 // Whole iterations of small grids, one launch each (fld_rows.cu): the tile of
 // rows a CTA owns (TJ = 0: the grid's rows do not fit), the kernel's
 // shared-memory attribute (call outside stream capture), and one iteration of
-// the FP32, hi/lo or float-float family from the buffers src (phi, D, phi lo)
-// into dst; with ghosts it also copies the ghost layer.
+// the FP32 or hi/lo family from the buffers src (phi, D, phi lo) into dst; the
+// first of a run also copies the ghost layer and is not launched early.
 struct RowsTile {
     int TJ, TK;
 };
 RowsTile rows_tile(const Layout &L, Family fam, int nsm);
 cudaError_t rows_prepare(Family fam, const PassParams &p);
 cudaError_t launch_rows(Family fam, const Layout &L, const Fields &f, const PassParams &p, const RowsTile &t,
-                        const float *const src[3], float *const dst[3], bool ghosts, cudaStream_t s);
+                        const float *const src[3], float *const dst[3], bool first, cudaStream_t s);
 
 // Relative residual Rbar / jbar of Eq. 37 from the device sums r2 = sum of
 // (R_p h^2)^2 over the unknowns at least `margin` voxels from the faces and

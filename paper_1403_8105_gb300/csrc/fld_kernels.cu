@@ -972,7 +972,8 @@ __global__ void __launch_bounds__(kPassDThreads) k_pass_d(Layout L, PassIndex ix
 // the caches), in strides of all CTAs.  One voxel per thread, the sums cost as
 // much as the residual itself and left one pair of partial sums per 256 voxels
 // for the last block to add: at 256^3 fresh D, residual and final sum took 104,
-// 362 and 79 us.
+// 362 and 79 us; now 108, 168 and 7 (the residual: 422 instructions a pair, issue 54 %
+// active, 72 registers; fresh D: 370 a pair, issue 73 %).
 constexpr int kCheckThreads = 128;
 constexpr int kCheckCtas = 2128;       // two waves of the residual's seven per SM of 152
 
@@ -1583,6 +1584,7 @@ cudaError_t launch_pdl(bool early, void (*k)(KArgs...), dim3 grd, dim3 blk, cuda
 constexpr long long kEarlyCtas = 912, kSettleCtas = 1216;
 bool pass_early(const PassParams &p, Family fam, dim3 g) {
     const long long ctas = (long long)g.x * g.y * g.z;
+    if (p.settle == 2) return false;
     if (fam != FAM_F64 && p.direct) return true;
     if (p.settle && ctas <= kSettleCtas) return false;
     const int asked = fam == FAM_F32 ? p.early_f32 : fam == FAM_FH ? p.early_fh : fam == FAM_FF ? p.early_ff : 1;

@@ -1,10 +1,9 @@
-// fld_rows.cu -- whole red-black iterations of small grids, one launch each
-// (sm_103a).
+// fld_rows.cu -- whole red-black iterations of the smallest grids, one launch
+// each (sm_103a).
 //
-// On a grid of 32^3 to 80^3 a launched colour pass (fld_kernels.cu) updates
-// 16 to 260 thousand unknowns: about 1.1 us of its 2 to 3 us is the step from
-// one launch to the next, and most of the rest one memory latency and one
-// chain of dependent operations.  Here one launch runs a whole iteration of
+// On a grid of 24^3 to 32^3 a launched colour pass (fld_kernels.cu) is little more
+// than the step from one launch to the next and one thread's chain of dependent
+// operations.  Here one launch runs a whole iteration of
 // Algorithm 1 (Koerner et al. 2014: the red pass, then the black one).  A CTA
 // owns TJ x TK rows (full in x).  It copies their state with a halo of two rows into
 // shared memory, updates the red unknowns of its rows and of the rows next to
@@ -13,9 +12,13 @@
 // its rows, and writes its rows to the other buffer of a ping-pong pair, so no
 // CTA reads what another writes in the same launch.  The medium does not
 // change: its rows are copied before the launch waits for the preceding one.
+// Half of its ~1300 instructions per warp (50^3) find addresses, and larger grids
+// repeat ever more red updates, so one pass per launch wins from 40^3 on, and in the
+// float-float family everywhere (us per iteration, hi/lo, passes / this: 24^3 3.5 / 2.8,
+// 32^3 3.7 / 3.3, 40^3 3.7 / 5.0).
 //
-// Every update is cell::cell_f32 / cell_fh / cell_ff, the code of the launched
-// passes, so the state is theirs bit for bit.  (The bfloat16 medium needs no
+// Every update is cell::cell_f32 / cell_fh, the code of the launched passes, so
+// the state is theirs bit for bit.  (The bfloat16 medium needs no
 // form of its own: sp and ah2 hold its values, exactly.)
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -157,12 +160,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_iter_rows(const RowsArgs a) {
         if (FAM == FAM_F32)
             cell_f32<LIM, ROUNDS, true>(own[it.o], ps, Ds, s_, ah, jj, lim, a.larsen_n, a.omega, a.inv2h, a.floor_,
                                         a.rounds, pn, dn);
-        else if (FAM == FAM_FH)
+        else
             cell_fh<LIM, ROUNDS, true>(own[it.o], own[2 * field + it.o], ps, ls, Ds, s_, ah, jj, lim, a.larsen_n,
                                        a.omega, a.inv2h, a.floor_, a.rounds, pn, ln, dn);
-        else
-            cell_ff<LIM, ROUNDS>(own[it.o], own[2 * field + it.o], ps, ls, Ds, s_, ah, jj, lim, a.larsen_n, a.omega,
-                                 a.inv2h, a.floor_, a.rounds, pn, ln, dn);
     };
     auto store = [&](int c, const Item &it, float pn, float dn, float ln) {
         if (c == 0 && it.write) {
@@ -245,7 +245,7 @@ RowsKernel pick(int lim, int rounds) {
 }
 
 RowsKernel rows_kernel(Family fam, int lim, int rounds) {
-    return fam == FAM_F32 ? pick<FAM_F32>(lim, rounds) : fam == FAM_FH ? pick<FAM_FH>(lim, rounds) : pick<FAM_FF>(lim, rounds);
+    return fam == FAM_F32 ? pick<FAM_F32>(lim, rounds) : pick<FAM_FH>(lim, rounds);
 }
 
 size_t rows_bytes(const Layout &L, int TJ, int TK, int nf) {
@@ -284,8 +284,8 @@ cudaError_t rows_prepare(Family fam, const PassParams &p) {
 }
 
 cudaError_t launch_rows(Family fam, const Layout &L, const Fields &f, const PassParams &p, const RowsTile &t,
-                        const float *const src[3], float *const dst[3], bool ghosts, cudaStream_t s) {
-    if (t.TJ < 1 || fam == FAM_F64) return cudaErrorInvalidValue;
+                        const float *const src[3], float *const dst[3], bool first, cudaStream_t s) {
+    if (t.TJ < 1 || (fam != FAM_F32 && fam != FAM_FH)) return cudaErrorInvalidValue;
     RowsArgs a;
     a.L = L;
     a.sp = f.sp; a.ah2 = f.ah2; a.jh2 = f.jh2;
@@ -307,7 +307,7 @@ cudaError_t launch_rows(Family fam, const Layout &L, const Fields &f, const Pass
     a.by_J2.set(t.TJ + 2);
     a.by_J.set(t.TJ);
     a.by_half.set(a.half);
-    a.ghosts = ghosts ? 1 : 0;
+    a.ghosts = first ? 1 : 0;
     a.lim = p.lim; a.rounds = p.local_iters;
     a.larsen_n = (float)p.larsen_n; a.omega = (float)p.omega; a.inv2h = (float)p.inv2h; a.floor_ = (float)p.floor_;
     cudaLaunchConfig_t cfg = {};
@@ -319,7 +319,7 @@ cudaError_t launch_rows(Family fam, const Layout &L, const Fields &f, const Pass
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = first ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, rows_kernel(fam, p.lim, p.local_iters), (const RowsArgs)a);
 }
 

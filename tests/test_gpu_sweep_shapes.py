@@ -40,7 +40,7 @@ def test_launched_passes_by_row_length(nx, precision, bf16):
 
 # Forms that the tuner picks on small grids, chosen here through a tuning cache
 # that names them: whole iterations per launch (-4), one unknown per thread (-5;
-# -2 in the float-float family).  Single rows and planes, rows whose first or last unknown is of
+# -2 in the float-float family, which has no -4).  Single rows and planes, rows whose first or last unknown is of
 # either colour, tiles cut at the far faces, an odd iteration left to the passes
 ROWS_SHAPES = [(1, 1, 1), (1, 1, 9), (9, 1, 6), (1, 40, 3), (2, 3, 2), (7, 9, 8), (17, 33, 31), (24, 24, 24),
                (32, 32, 32), (40, 37, 33), (5, 6, 250)]
@@ -71,7 +71,7 @@ def test_small_grid_forms_equal_the_pair_passes(tmp_path, form):
 
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     lines = ["v6 %dx%dx%d fam%d lim%d r2 bf%d sm%d | %d 1 64 0 0 0"
-             % (s[2], s[1], s[0], fam, lim, bf, sms, -2 if form == -5 and fam == 1 else form)
+             % (s[2], s[1], s[0], fam, lim, bf, sms, -2 if fam == 1 else form)
              for s in ROWS_SHAPES for fam in (0, 1, 3) for lim in (fld.LIMITERS["lp"], fld.LIMITERS["larsen"])
              for bf in (0, 1)]
     cache = tmp_path / "tune.txt"
