@@ -1579,14 +1579,16 @@ cudaError_t launch_pdl(bool early, void (*k)(KArgs...), dim3 grd, dim3 blk, cuda
 // (6.1 / 5.4 / 8.0); 4, 16 and 32 launches differ by 3 %.  From 80^3 on all early is as fast
 // or faster (96^3 7.7 against 7.9).  Otherwise as asked by the tuner, or (-1) if there
 // are more than six CTAs per SM.  Launches that do not come from a graph are 4 us apart
-// unless early, which is worse than any placement; FP64 passes take longer than that
+// unless early: those only settle (256 iterations of 54^3 FP32 through fld_iterate, us
+// each: 6.1 all early, 4.7; start 6.0), up to a size at which it costs more than it saves
+// (80^3 hi/lo 7.5, settled 8.1); FP64 passes take longer than that
 // (32^3, a pass in a graph: all early 20 us, never 9.9, settled 9.7).
 constexpr long long kEarlyCtas = 912, kSettleCtas = 1216;
 bool pass_early(const PassParams &p, Family fam, dim3 g) {
     const long long ctas = (long long)g.x * g.y * g.z;
     if (p.settle == 2) return false;
+    if (p.settle && ctas <= (p.direct ? kEarlyCtas : kSettleCtas)) return false;
     if (fam != FAM_F64 && p.direct) return true;
-    if (p.settle && ctas <= kSettleCtas) return false;
     const int asked = fam == FAM_F32 ? p.early_f32 : fam == FAM_FH ? p.early_fh : fam == FAM_FF ? p.early_ff : 1;
     return asked >= 0 ? asked != 0 : ctas > kEarlyCtas;
 }
@@ -1601,6 +1603,10 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
         const dim3 g1 = item_grid(L, (L.nx + 1) / 2, true, &ix);
         auto k = fam == FAM_FH ? k_pass1<-1, 0, true> : k_pass1<-1, 0, false>;
         if (p.local_iters == 2 && p.lim == LIM_LP) k = fam == FAM_FH ? k_pass1<LIM_LP, 2, true> : k_pass1<LIM_LP, 2, false>;
+        else if (p.local_iters == 2 && p.lim == LIM_KERSHAW)
+            k = fam == FAM_FH ? k_pass1<LIM_KERSHAW, 2, true> : k_pass1<LIM_KERSHAW, 2, false>;
+        else if (p.local_iters == 2 && p.lim == LIM_LARSEN)
+            k = fam == FAM_FH ? k_pass1<LIM_LARSEN, 2, true> : k_pass1<LIM_LARSEN, 2, false>;
         return launch_pdl(pass_early(p, fam, g1), k, g1, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.phi,
                           f.phlo, f.D, colour, p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h,
                           (float)p.floor_, p.local_iters);
