@@ -648,8 +648,10 @@ void set_valid(fld_grid_s *g, Family fam) {
 
 // ---------------------------------------------------------------------------
 // Autotuner (not a paper item): for each grid shape, sweep family, limiter and
-// medium it times the launched colour passes against every blocked
-// configuration on the grid itself, and the residual check against one
+// medium it times the forms of the launched colour passes (pairs, quads; on
+// small grids one unknown per thread, whole iterations, and both launch
+// policies) and every blocked configuration on the grid itself, replayed from
+// graphs as a solve replays them, and the residual check against one
 // iteration, and keeps
 //   * the fastest sweep launch shape (all of them give the same bits, so the
 //     choice changes the time only), and
@@ -745,6 +747,15 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
     fa.phi = g->alt_phi;
     fa.D = g->alt_D;
     fa.phlo = g->alt_lo;
+    // captured on a stream of its own: the grid's may be the legacy default
+    // stream, which cannot be captured, or one that another thread uses
+    struct CaptureStream {
+        cudaStream_t s = nullptr;
+        ~CaptureStream() {
+            if (s) cudaStreamDestroy(s);
+        }
+    } cap;
+    FLD_CK(cudaStreamCreateWithFlags(&cap.s, cudaStreamNonBlocking));
     const int n = 16;   // iterations per timing, a multiple of every depth
     TuneChoice c;
     double best = INFINITY;
@@ -770,23 +781,23 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
                 const float *const a[3] = {g->f.phi, g->f.D, g->f.phlo};
                 float *const b[3] = {g->alt_phi, g->alt_D, g->alt_lo};
                 for (int it = 0; it < n && e == cudaSuccess; ++it)
-                    e = launch_rows(fam, g->L, g->f, pc, g->rtile[rows_slot(fam)], a, b, it == 0, g->stream);
+                    e = launch_rows(fam, g->L, g->f, pc, g->rtile[rows_slot(fam)], a, b, it == 0, cap.s);
             } else if (cand < 0) {
                 for (int it = 0; it < 2 * n && e == cudaSuccess; ++it) {
                     pc.settle = it % kSettleEvery == 0;
-                    e = launch_pass(fam, g->L, fa, pc, it & 1, g->stream);
+                    e = launch_pass(fam, g->L, fa, pc, it & 1, cap.s);
                 }
             } else {
                 for (int i = 0; i < n / tiled_depth(cand) && e == cudaSuccess; ++i)
                     e = launch_tiled(fam, cand, g->L, g->f, pp, g->maps[cand][0], g->alt_phi, g->alt_D, g->alt_lo,
-                                     g->tiled_status, g->nsm, g->stream);
+                                     g->tiled_status, g->nsm, cap.s);
             }
             return e;
         };
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
-        FLD_CK(cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal));
-        const cudaError_t e1 = iterate(), e2 = cudaStreamEndCapture(g->stream, &graph);
+        FLD_CK(cudaStreamBeginCapture(cap.s, cudaStreamCaptureModeThreadLocal));
+        const cudaError_t e1 = iterate(), e2 = cudaStreamEndCapture(cap.s, &graph);
         cudaError_t ce = e1 != cudaSuccess ? e1 : e2;
         if (ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, graph, 0);
         if (graph) cudaGraphDestroy(graph);

@@ -86,3 +86,22 @@ def test_small_grid_forms_equal_the_pair_passes(tmp_path, form):
     for key in got.files:
         if " 0 " in key:
             assert np.array_equal(got[key], got[key.replace(" 0 ", " -1 ")]), key
+
+
+# Every family the tuner times, on the legacy default stream (handle 1), which
+# cannot be captured: shapes that nothing else here has tuned
+@pytest.mark.parametrize("precision,shape", [("fp32", (6, 13, 19)), ("pair", (6, 13, 21)), ("mixed", (6, 13, 23))])
+def test_tuning_on_the_legacy_stream(precision, shape):
+    sig, alb, j, h = random_case(shape, 31)
+    want = state_after(shape, precision, -1, 5)
+    rng = np.random.default_rng(31)
+    padded = tuple(n + 2 for n in shape)
+    phi0, D0 = rng.uniform(0.05, 1.5, padded), rng.uniform(0.0, 0.1, padded)
+    nz, ny, nx = shape
+    with fld.Grid(nx, ny, nz, h, stream=1) as g:
+        g.set_medium(sig, alb)
+        g.set_source(j)
+        g.set_state(phi0, D0)
+        g.iterate(fld.params(limiter="lp", precision=precision, omega=1.4, warm_start=1), 5)
+        got = g.get_state()
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
