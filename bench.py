@@ -62,7 +62,7 @@ BYTES_PER_UPDATE = {"fp32": 28, "fh": 28, "ff": 28}
 BYTES_PER_UPDATE_BF16 = {"fp32": 24, "fh": 24, "ff": 28}
 KERNEL_NAME = {"fp32": "k_pass2_f32 (single-precision red/black pass, two unknowns per thread)",
                "fh": "k_pass2_fh (hi/lo phi, FP32-summed red/black pass, two unknowns per thread)",
-               "ff": "k_pass_ff (float-float correction pass)"}
+               "ff": "k_pass2_ff (float-float correction pass, two unknowns per thread)"}
 
 
 def parse_args():
@@ -1241,8 +1241,6 @@ def run_sweeps(args):
                         ach = 28.0 * n ** 3 / (us * 1e-6) / 1e9
                         if depth >= 0:
                             name = f"blocked T={depth}"
-                        elif fam == "ff":
-                            name = "launched, 1 unknown per thread"
                         else:
                             name = f"launched, {cells} unknowns per thread"
                         out[f"{n} {fam} {name}"] = {

@@ -210,10 +210,12 @@ typedef struct {
                              0 (default): chosen per grid shape, sweep family,
                              limiter and medium by the library's autotuner,
                              which times the launched passes (2 and 4 unknowns
-                             per thread) and every blocked configuration on the
-                             grid itself the first time that combination is
-                             solved, keeps the fastest for the process and
-                             appends it to a cache file (FLD_TUNE_CACHE, else
+                             per thread; on small grids also 1, whole iterations
+                             per launch, and launches that wait for one another)
+                             and every blocked configuration on the grid itself
+                             the first time that combination is solved, keeps
+                             the fastest for the process and appends it to a
+                             cache file (FLD_TUNE_CACHE, else
                              fld_tune_cache.txt beside the library).  The
                              choice changes the time only, not the result.
                              Not in the paper.                                 */
