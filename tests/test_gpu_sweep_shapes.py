@@ -105,3 +105,43 @@ def test_tuning_on_the_legacy_stream(precision, shape):
         g.iterate(fld.params(limiter="lp", precision=precision, omega=1.4, warm_start=1), 5)
         got = g.get_state()
     assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+
+
+# Ticks: the third and later calls of fld_iterate with one count and set of
+# parameters replay a graph on a small grid; a changed count or parameter, a
+# state set between the calls, a caller's own capture and the legacy stream
+# leave the bits of plain launches (temporal_depth -1 on a grid of its own each)
+@pytest.mark.parametrize("precision,bf16", [("fp32", 0), ("pair", 1), ("mixed", 0)])
+@pytest.mark.parametrize("legacy", [0, 1])
+def test_repeated_iterate_replays_the_same_bits(precision, bf16, legacy):
+    shape = (11, 14, 37)
+    sig, alb, j, h = random_case(shape, 7)
+    rng = np.random.default_rng(7)
+    padded = tuple(n + 2 for n in shape)
+    states = [(rng.uniform(0.05, 1.5, padded), rng.uniform(0.0, 0.1, padded)) for _ in range(2)]
+    nz, ny, nx = shape
+
+    def par(omega, depth):
+        return fld.params(precision=precision, omega=omega, warm_start=1, temporal_depth=depth, medium_bf16=bf16)
+
+    stream = torch.cuda.Stream()
+    with fld.Grid(nx, ny, nz, h, stream=1 if legacy else stream.cuda_stream) as g, gpu_grid(sig, alb, j, h) as ref:
+        g.set_medium(sig, alb)
+        g.set_source(j)
+        calls = [(5, 1.4)] * 5 + [(6, 1.4)] * 4 + [(6, 1.2)] * 4 + [(5, 1.4)] * 3
+        for s, (phi0, D0) in enumerate(states):
+            g.set_state(phi0, D0)
+            ref.set_state(phi0, D0)
+            for n, omega in calls:
+                g.iterate(par(omega, 0), n)
+                ref.iterate(par(omega, -1), n)
+        if not legacy:
+            torch.cuda.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+                g.iterate(par(1.4, 0), 5)
+            graph.replay()
+            torch.cuda.synchronize()
+            ref.iterate(par(1.4, -1), 5)
+        got, want = g.get_state(), ref.get_state()
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
