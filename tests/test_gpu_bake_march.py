@@ -44,3 +44,16 @@ def test_point(shape, where):
         g.bake_point(pos, 3.0)
         got = g.get_source()
     assert np.abs(got - want).max() <= TOL * np.abs(want).max()
+
+
+# steps so short that the count of samples is kept in whole numbers (2^20 of them
+# span less than twice the longest axis), against steps a little longer, which
+# count in float: the two depths differ by rounding only
+def test_sample_count_forms():
+    sig, alb, j, h = random_case((2, 3, 2), 5)
+    got = []
+    for step in (5.6e-6, 5.8e-6):
+        with gpu_grid(sig, alb, j, h) as g:
+            g.bake_directional((0.2, 0.9, 0.1), 1.5, step * h)
+            got.append(g.get_source())
+    assert np.abs(got[0] - got[1]).max() <= TOL * np.abs(got[1]).max()
