@@ -1362,10 +1362,16 @@ __device__ __forceinline__ float sigma_at(const float *__restrict__ st, const Ma
 }
 
 // Where the light is, in voxels: the unit direction towards it, or its position.
+// Beyond kFarLight (of a voxel, or of the world's unit) squares near the end of
+// the range of a float; beyond kFarthest the host scales the position nearer,
+// where the direction from every voxel is the same to the last bit.
+constexpr float kFarLight = 1e18f;
+constexpr double kFarthest = 1e30;
 struct MarchLight {
     float w[3], pos[3];
     int point;
     float value, step, h;
+    float unit;                  // world length of a unit of pos: h, unless the light is scaled nearer
 };
 
 template <bool WIDE>
@@ -1387,11 +1393,19 @@ __global__ void __launch_bounds__(256) k_bake_march(Layout L, const float *__res
     float w[3] = {m.w[0], m.w[1], m.w[2]};
     float r = 0.0f;
     if (m.point) {
-        const float d[3] = {m.pos[0] - x[0], m.pos[1] - x[1], m.pos[2] - x[2]};
+        float d[3] = {m.pos[0] - x[0], m.pos[1] - x[1], m.pos[2] - x[2]};
+        // for a light so far that the squares overflow the march would find neither
+        // direction nor end (2^31 samples): the components go relative to the largest
+        const float most = fmaxf(fmaxf(fabsf(d[0]), fabsf(d[1])), fabsf(d[2]));
+        const float scale = most > kFarLight ? most : 1.0f;
+        if (most > kFarLight) {
+            d[0] /= scale; d[1] /= scale; d[2] /= scale;
+        }
         r = sqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
         if (r > 0.0f) {
             w[0] = d[0] / r; w[1] = d[1] / r; w[2] = d[2] / r;
         }
+        r *= scale;
     }
     float len = INFINITY;
     MarchAxis ax[3];
@@ -1429,8 +1443,9 @@ __global__ void __launch_bounds__(256) k_bake_march(Layout L, const float *__res
     }
     float e = m.value * scatter * transmittance(ff_mul_f(tau, m.h));
     if (m.point) {
-        const float rr = fmaxf(r, 0.5f) * m.h;
-        e = e / (4.0f * 3.14159265358979f * rr * rr);
+        const float rr = fmaxf(r, 0.5f) * m.unit;
+        const float area = 4.0f * 3.14159265358979f * rr;
+        e = rr > kFarLight ? e / area / rr : e / (area * rr);
     }
     js[v] = accumulate ? js[v] + e : e;
 }
@@ -1854,8 +1869,11 @@ cudaError_t launch_bake_march(const Layout &L, const Fields &f, double h, const 
     MarchLight m;
     for (int a = 0; a < 3; ++a) {
         m.w[a] = (float)w[a];
-        m.pos[a] = (float)(pos[a] / h - 0.5);
     }
+    double far = 0.0;            // of the light, in voxels and units of kFarthest
+    for (int a = 0; a < 3; ++a) far = fmax(far, fabs(pos[a]) / kFarthest / h);
+    for (int a = 0; a < 3; ++a) m.pos[a] = (float)(far > 1.0 ? pos[a] / far / h : pos[a] / h - 0.5);
+    m.unit = (float)(far > 1.0 ? h * far : h);
     m.point = point;
     m.value = value;
     m.step = (float)(step / h < 1e30 ? step / h : 1e30);
