@@ -1320,6 +1320,11 @@ __device__ __forceinline__ float lower_corner(const MarchAxis &a, float &u, int 
     return u - (float)b;
 }
 
+// Two instructions, as a + f (b - a) takes, but exact at both ends and never off by
+// more than two roundings of the result: that one reads 9.77e-4 at f = 1 between
+// 1e4 and 1e-3, the rounding of the dense side.
+__device__ __forceinline__ float blend(float f, float a, float b) { return fmaf(f, b, fmaf(-f, a, a)); }
+
 template <bool WIDE>
 __device__ __forceinline__ float sigma_at(const float *__restrict__ st, const MarchAxis ax[3], const int sy, const int sz,
                                           const int bias, float ux, float uy, float uz) {
@@ -1355,10 +1360,8 @@ __device__ __forceinline__ float sigma_at(const float *__restrict__ st, const Ma
     const int dx = WIDE ? ax[0].stride : 1;
     const float a0 = __ldg(p), a1 = __ldg(p + dx), b0 = __ldg(py), b1 = __ldg(py + dx);
     const float c0 = __ldg(pz), c1 = __ldg(pz + dx), d0 = __ldg(pyz), d1 = __ldg(pyz + dx);
-    const float a = fmaf(fx, a1 - a0, a0), b = fmaf(fx, b1 - b0, b0);
-    const float c = fmaf(fx, c1 - c0, c0), d = fmaf(fx, d1 - d0, d0);
-    const float e = fmaf(fy, b - a, a), f = fmaf(fy, d - c, c);
-    return fmaf(fz, f - e, e);
+    const float a = blend(fx, a0, a1), b = blend(fx, b0, b1), c = blend(fx, c0, c1), d = blend(fx, d0, d1);
+    return blend(fz, blend(fy, a, b), blend(fy, c, d));
 }
 
 // Where the light is, in voxels: the unit direction towards it, or its position.
