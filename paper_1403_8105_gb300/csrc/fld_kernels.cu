@@ -1426,17 +1426,27 @@ __global__ void __launch_bounds__(256) k_bake_march(Layout L, const float *__res
     const uint32_t mb = (uint32_t)__float_as_int(kRound);
     const int bias = (int)(4u * (mb * (uint32_t)sz + mb * (uint32_t)sy + mb));
     // sum of the samples in float-float: TwoSum, the errors in a word of their own
+    // that every fourth sample folds back (left to grow, its own rounding reached 9e-7 of
+    // the sum over 1e5 equal samples)
     ff sum = {0.0f, 0.0f};
     const int m_full = (int)floorf(len / m.step);
     float mid = 0.5f;            // q + 1/2 (exact; WIDE takes marches of over 2^20 steps)
-    for (int q = 0; q < m_full; ++q, mid += 1.0f) {
+    auto sample = [&](int q) {
         const float t = (WIDE ? (float)q + 0.5f : mid) * m.step;
+        mid += 1.0f;
         const float s = sigma_at<WIDE>(st, ax, sy, sz, bias, fmaf(t, w[0], x[0]), fmaf(t, w[1], x[1]),
                                        fmaf(t, w[2], x[2]));
         const ff u = two_sum(sum.hi, s);
         sum.hi = u.hi;
         sum.lo = __fadd_rn(sum.lo, u.lo);
+    };
+    int q = 0;
+    for (; q < m_full - 3; q += 4) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) sample(q + u);
+        sum = fast_two_sum(sum.hi, sum.lo);
     }
+    for (; q < m_full; ++q) sample(q);
     ff tau = ff_mul_f(fast_two_sum(sum.hi, sum.lo), m.step);
     const float rem = len - (float)m_full * m.step;
     if (rem > 1e-6f * m.step) {
