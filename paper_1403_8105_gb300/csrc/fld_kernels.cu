@@ -956,8 +956,8 @@ __global__ void __launch_bounds__(kPassDThreads) k_pass_d(Layout L, PassIndex ix
         }
         const double N = fma(0.5 * P, A, base * Q), W = fma(3.0, P, den0 * Q);
         const double both = 1.0 / (Q * W);
-        delta = N * Q * both;
-        Dp = P * W * both;
+        delta = N * (Q * both);     // (P W overflows where sigma' is below 1e-154)
+        Dp = P * (W * both);
     }
     phi[o.own] = fma(omega, delta, p0);
     D[o.own] = Dp;
