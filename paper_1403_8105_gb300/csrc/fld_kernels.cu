@@ -53,29 +53,6 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
     return r;
 }
 
-// Sum over the block of a float-float value per thread, valid in thread 0:
-// float-float shuffles within each warp, then the warps' sums in FP64 in
-// warp order (GB300's FP64 rate is a small fraction of its FP32 rate, so the
-// per-element sums stay on the FP32 pipes).
-__device__ __forceinline__ double block_sum_ff(ff v, double *sh) {
-    const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-    const int nthr = blockDim.x * blockDim.y * blockDim.z;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const ff u{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)};
-        v = ff_add(v, u);
-    }
-    __syncthreads();
-    if ((tid & 31) == 0) sh[tid >> 5] = ff_to_d(v);
-    __syncthreads();
-    double r = 0.0;
-    if (tid < 32) {
-        r = (tid < (nthr + 31) / 32) ? sh[tid] : 0.0;
-        r = warp_sum(r);
-    }
-    return r;
-}
-
 // Second pass: fixed-order sum of the per-block partial pairs.
 __global__ void __launch_bounds__(kRedThreads) k_finalize(const double *__restrict__ partials, int nblocks,
                                                          double *__restrict__ result) {
@@ -1036,18 +1013,59 @@ __global__ void k_fresh_D_d(Layout L, const double *__restrict__ sp, const doubl
                         phi[L.at(i, j, k + 1)] - phi[L.at(i, j, k - 1)], inv2h, sp[q], phi[q], floor_, lim, larsen_n);
 }
 
+// The two running sums of a residual check (in x and y) in three words each: every
+// TwoSum's error is added to the next word, so that hundreds of terms a thread
+// leave no more than one does. (By float-float additions 980 equal terms, whose
+// roundings do not cancel, were 7e-13 off.) Packed, the two cost what two
+// float-float additions did.
+struct Sums {
+    float2 hi, lo, err;
+};
+__device__ __forceinline__ void sums_add(Sums &s, ff2 x) {
+    const ff2 t = two_sum2(s.hi, x.hi), u = two_sum2(s.lo, t.lo), v = two_sum2(u.hi, x.lo);
+    s.hi = t.hi;
+    s.lo = v.hi;
+    s.err = add2(s.err, add2(u.lo, v.lo));
+}
+
+// Their sums over the CTA, into its pair of partials: shuffles within each warp,
+// then the warps' sums in FP64 in warp order (GB300's FP64 rate is a small
+// fraction of its FP32 rate, so the per-element sums stay on the FP32 pipes).
+__device__ __forceinline__ void store_partials(Sums v, double *__restrict__ p) {
+    __shared__ double sh[2][kCheckThreads / 32];
+    auto down = [](float2 a, int o) {
+        return make_float2(__shfl_down_sync(0xffffffffu, a.x, o), __shfl_down_sync(0xffffffffu, a.y, o));
+    };
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const ff2 u{down(v.hi, o), down(v.lo, o)};
+        const float2 e = down(v.err, o);
+        sums_add(v, u);
+        v.err = add2(v.err, e);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        sh[0][threadIdx.x >> 5] = (double)v.hi.x + ((double)v.lo.x + (double)v.err.x);
+        sh[1][threadIdx.x >> 5] = (double)v.hi.y + ((double)v.lo.y + (double)v.err.y);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double a = 0.0;
+#pragma unroll
+        for (int w = 0; w < kCheckThreads / 32; ++w) a += sh[threadIdx.x][w];
+        p[threadIdx.x] = a;
+    }
+}
+
 // Residual R_p dl^2 = jh2 - ah2 phi_p + sum_s D_ps (phi_s - phi_p) in
 // float-float (packed, as the correction pass forms it): per thread the sums of
-// its square over the margin set and of the source's square over all unknowns,
-// in float-float.
+// its square over the margin set and of the source's square over all unknowns.
 template <bool LO>
 __device__ __forceinline__ void residual_pairs(const Layout &L, const CheckIndex &ix, int cta, int ctas,
                                                const float *__restrict__ ah2, const float *__restrict__ jh2,
                                                const float *__restrict__ phi, const float *__restrict__ phlo,
                                                const float *__restrict__ Df, const float *__restrict__ Dghost,
-                                               int margin, ff &r2, ff &j2) {
-    r2 = ff{0.0f, 0.0f};
-    j2 = ff{0.0f, 0.0f};
+                                               int margin, Sums &sums) {
+    sums = Sums{both(0.0f), both(0.0f), both(0.0f)};
     for_pairs(L, ix, cta, ctas, [&](const Pair &q, int c, int t, int J, int K) {
         float2 ps[6], ls[6], Ds[6];
         gather_packed(phi, q, ps);
@@ -1070,25 +1088,16 @@ __device__ __forceinline__ void residual_pairs(const Layout &L, const CheckIndex
         const ff2 S = ff_S_pair(T, ld2(Df, q.own));
         const ff sx{S.hi.x, S.lo.x}, sy{S.hi.y, S.lo.y};
         const bool in = J > margin && J <= L.ny - margin && K > margin && K <= L.nz - margin;
-        if (in && I0 > margin && I0 <= L.nx - margin) r2 = ff_add(r2, ff_mul(sx, sx));
-        j2 = ff_add(j2, two_prod(jj.x, jj.x));
+        ff r0{0.0f, 0.0f}, r1{0.0f, 0.0f}, j0 = two_prod(jj.x, jj.x), j1{0.0f, 0.0f};
+        if (in && I0 > margin && I0 <= L.nx - margin) r0 = ff_mul(sx, sx);
         if (q.second) {
-            if (in && I0 + 2 > margin && I0 + 2 <= L.nx - margin) r2 = ff_add(r2, ff_mul(sy, sy));
-            j2 = ff_add(j2, two_prod(jj.y, jj.y));
+            if (in && I0 + 2 > margin && I0 + 2 <= L.nx - margin) r1 = ff_mul(sy, sy);
+            j1 = two_prod(jj.y, jj.y);
         }
+        // the pair's two terms first (ff_add)
+        const ff2 two = two_sum2(make_float2(r0.hi, j0.hi), make_float2(r1.hi, j1.hi));
+        sums_add(sums, fast_two_sum2(two.hi, add2(two.lo, add2(make_float2(r0.lo, j0.lo), make_float2(r1.lo, j1.lo)))));
     });
-}
-
-// The CTA's sums into its pair of partials.
-__device__ __forceinline__ void store_partials(ff r2f, ff j2f, double *__restrict__ p) {
-    __shared__ double sh[32];
-    const double r2 = block_sum_ff(r2f, sh);
-    __syncthreads();
-    const double j2 = block_sum_ff(j2f, sh);
-    if (threadIdx.x == 0) {
-        p[0] = r2;
-        p[1] = j2;
-    }
 }
 
 __global__ void __launch_bounds__(kCheckThreads) k_residual_f(Layout L, CheckIndex ix, const float *__restrict__ ah2,
@@ -1098,10 +1107,10 @@ __global__ void __launch_bounds__(kCheckThreads) k_residual_f(Layout L, CheckInd
                                                                const float *__restrict__ Df,
                                                                const float *__restrict__ Dghost, int margin,
                                                                double *__restrict__ partials) {
-    ff r2, j2;
-    if (phlo) residual_pairs<true>(L, ix, blockIdx.x, gridDim.x, ah2, jh2, phi, phlo, Df, Dghost, margin, r2, j2);
-    else residual_pairs<false>(L, ix, blockIdx.x, gridDim.x, ah2, jh2, phi, phlo, Df, Dghost, margin, r2, j2);
-    store_partials(r2, j2, partials + 2 * (long long)blockIdx.x);
+    Sums sums;
+    if (phlo) residual_pairs<true>(L, ix, blockIdx.x, gridDim.x, ah2, jh2, phi, phlo, Df, Dghost, margin, sums);
+    else residual_pairs<false>(L, ix, blockIdx.x, gridDim.x, ah2, jh2, phi, phlo, Df, Dghost, margin, sums);
+    store_partials(sums, partials + 2 * (long long)blockIdx.x);
 }
 
 // Batched fresh D / residual / finalize: CTA b works on grid cta_grid[b] as CTA
@@ -1124,10 +1133,10 @@ __global__ void __launch_bounds__(kCheckThreads) k_residual_batch(const BatchDes
     const BatchDesc d = load_desc(descs + __ldg(cta_grid + blockIdx.x));
     if (!d.active) return;
     const int local = blockIdx.x - d.res_first;
-    ff r2, j2;
-    if (d.mode) residual_pairs<true>(d.L, d.ix, local, d.res_n, d.ah2, d.jh2, d.phi, d.phlo, d.Df, d.D, margin, r2, j2);
-    else residual_pairs<false>(d.L, d.ix, local, d.res_n, d.ah2, d.jh2, d.phi, d.phlo, d.Df, d.D, margin, r2, j2);
-    store_partials(r2, j2, partials + 2 * (long long)(d.res_slot + local));
+    Sums sums;
+    if (d.mode) residual_pairs<true>(d.L, d.ix, local, d.res_n, d.ah2, d.jh2, d.phi, d.phlo, d.Df, d.D, margin, sums);
+    else residual_pairs<false>(d.L, d.ix, local, d.res_n, d.ah2, d.jh2, d.phi, d.phlo, d.Df, d.D, margin, sums);
+    store_partials(sums, partials + 2 * (long long)(d.res_slot + local));
 }
 
 __global__ void __launch_bounds__(kRedThreads) k_finalize_batch(const BatchDesc *__restrict__ descs,
