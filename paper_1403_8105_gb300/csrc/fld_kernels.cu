@@ -718,6 +718,9 @@ __global__ void __launch_bounds__(kMultiThreadsX * kMultiThreadsY, 4)
             tile_f32<LIM, ROUNDS, BF>(d.L, d.sp, d.ah2, d.jh2, d.spb, d.sab, d.h2, d.phi, d.D, colour, d.lim,
                                       d.larsen_n, d.omega, d.inv2h, d.floor_, d.local_iters, t, J, bz + 1);
     }
+    // a table of one-voxel grids has passes without unknowns: one CTA waits all the
+    // same, so that the pass does not end before the preceding one
+    if (blockIdx.x == 0) pdl_wait();
 }
 
 template <bool BF, bool HL>
@@ -1631,10 +1634,12 @@ cudaError_t launch_pdl(bool early, void (*k)(KArgs...), dim3 grd, dim3 blk, cuda
 // each: 6.1 all early, 4.7; start 6.0), up to a size at which it costs more than it saves
 // (80^3 hi/lo 7.5, settled 8.1); FP64 passes take longer than that
 // (32^3, a pass in a graph: all early 20 us, never 9.9, settled 9.7).
+// A grid of one voxel is never early: no thread of its black pass has an unknown, so
+// none waits for the red pass, and the next one would follow an empty pass alone.
 constexpr long long kEarlyCtas = 912, kSettleCtas = 1216;
-bool pass_early(const PassParams &p, Family fam, dim3 g) {
+bool pass_early(const PassParams &p, Family fam, const Layout &L, dim3 g) {
     const long long ctas = (long long)g.x * g.y * g.z;
-    if (p.settle == 2) return false;
+    if (p.settle == 2 || (L.nx == 1 && L.ny == 1 && L.nz == 1)) return false;
     if (p.settle && ctas <= (p.direct ? kEarlyCtas : kSettleCtas)) return false;
     if (fam != FAM_F64 && p.direct) return true;
     const int asked = fam == FAM_F32 ? p.early_f32 : fam == FAM_FH ? p.early_fh : fam == FAM_FF ? p.early_ff : 1;
@@ -1655,7 +1660,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
             k = fam == FAM_FH ? k_pass1<LIM_KERSHAW, 2, true> : k_pass1<LIM_KERSHAW, 2, false>;
         else if (p.local_iters == 2 && p.lim == LIM_LARSEN)
             k = fam == FAM_FH ? k_pass1<LIM_LARSEN, 2, true> : k_pass1<LIM_LARSEN, 2, false>;
-        return launch_pdl(pass_early(p, fam, g1), k, g1, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.phi,
+        return launch_pdl(pass_early(p, fam, L, g1), k, g1, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.phi,
                           f.phlo, f.D, colour, p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h,
                           (float)p.floor_, p.local_iters);
     }
@@ -1669,7 +1674,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
                 constexpr bool B = decltype(bf)::value, H = decltype(hl)::value;
                 auto k = k_pass4<-1, 0, B, H>;
                 if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass4<LIM_LP, 2, B, H>;
-                return launch_pdl(pass_early(p, fam, grd4), k, grd4, blk4, s, L, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
+                return launch_pdl(pass_early(p, fam, L, grd4), k, grd4, blk4, s, L, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
                                   f.D, colour, p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h,
                                   (float)p.floor_, p.local_iters);
             };
@@ -1687,7 +1692,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
             else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_f32<LIM_LARSEN, 2, B, R>;
             PassIndex ix;
             const dim3 g2 = item_grid(L, pairs, R, &ix);
-            return launch_pdl(pass_early(p, fam, g2), k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.D, colour,
+            return launch_pdl(pass_early(p, fam, L, g2), k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.D, colour,
                               p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_,
                               p.local_iters);
         };
@@ -1706,7 +1711,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
             if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass_ff<LIM_LP, 2>;
             else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass_ff<LIM_KERSHAW, 2>;
             else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass_ff<LIM_LARSEN, 2>;
-            return launch_pdl(pass_early(p, fam, grd), k, grd, blk, s, L, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour, p.lim,
+            return launch_pdl(pass_early(p, fam, L, grd), k, grd, blk, s, L, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour, p.lim,
                               (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_, p.local_iters);
         }
         auto pick = [&](auto run) {
@@ -1718,7 +1723,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
                         ? k_pass2_ff<LIM_LP, 2, R, 5> : k_pass2_ff<LIM_LP, 2, R, 7>;
             else if (p.local_iters == 2 && p.lim == LIM_KERSHAW) k = k_pass2_ff<LIM_KERSHAW, 2, R, 7>;
             else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_ff<LIM_LARSEN, 2, R, 7>;
-            return launch_pdl(pass_early(p, fam, g2), k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour,
+            return launch_pdl(pass_early(p, fam, L, g2), k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.phi, f.phlo, f.D, colour,
                               p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h, (float)p.floor_,
                               p.local_iters);
         };
@@ -1733,7 +1738,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
             else if (p.local_iters == 2 && p.lim == LIM_LARSEN) k = k_pass2_fh<LIM_LARSEN, 2, B, R>;
             PassIndex ix;
             const dim3 g2 = item_grid(L, pairs, R, &ix);
-            return launch_pdl(pass_early(p, fam, g2), k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
+            return launch_pdl(pass_early(p, fam, L, g2), k, g2, dim3(kPassThreads), s, L, ix, f.sp, f.ah2, f.jh2, f.spb, f.sab, (float)p.h2, f.phi, f.phlo,
                               f.D, colour, p.lim, (float)p.larsen_n, (float)p.omega, (float)p.inv2h,
                               (float)p.floor_, p.local_iters);
         };
@@ -1748,7 +1753,7 @@ cudaError_t launch_pass(Family fam, const Layout &L, const Fields &f, const Pass
         auto k = k_pass_d<-1, 0>;
         if (p.local_iters == 2 && p.lim == LIM_LP) k = k_pass_d<LIM_LP, 2>;
         const dim3 gd((ix.total + kPassDThreads - 1) / kPassDThreads);
-        return launch_pdl(pass_early(p, fam, gd), k, gd, dim3(kPassDThreads), s, L, ix,
+        return launch_pdl(pass_early(p, fam, L, gd), k, gd, dim3(kPassDThreads), s, L, ix,
                           f.sp64, f.ah264, f.jh264, f.phi64, f.D64, colour, p.lim, p.larsen_n, p.omega, p.inv2h,
                           p.floor_, p.local_iters);
         }
