@@ -2159,18 +2159,20 @@ fld_status server_workspace(fld_server_s *s, int grids, int res) {
     return FLD_OK;
 }
 
-// Room for the Anderson dot products of `grids` grids.
+// Room for the Anderson dot products of `grids` grids, made as a grid joins: a step
+// that failed for want of it would leave its decisions half taken.  The room there
+// was is kept until there is more.
 fld_status server_dots(fld_server_s *s, int grids) {
     if (s->p.anderson <= 0 || grids <= s->cap_dots) return FLD_OK;
     FLD_CK(cudaStreamSynchronize(s->bs));
-    if (s->d_dots) cudaFree(s->d_dots);
-    s->d_dots = nullptr;
-    s->cap_dots = 0;
     const int cap = grids + grids / 2 + 4;
-    if (cudaMalloc((void **)&s->d_dots, sizeof(double) * kAndersonMax * (size_t)cap) != cudaSuccess) {
+    double *more = nullptr;
+    if (cudaMalloc((void **)&more, sizeof(double) * kAndersonMax * (size_t)cap) != cudaSuccess) {
         (void)cudaGetLastError();
         return fail(FLD_ERR_OOM, "cudaMalloc of the dot products failed");
     }
+    if (s->d_dots) cudaFree(s->d_dots);
+    s->d_dots = more;
     s->cap_dots = cap;
     return FLD_OK;
 }
@@ -2202,6 +2204,16 @@ cudaError_t server_join(fld_server_s *s, size_t nside) {
     }
     return cudaSuccess;
 }
+
+// A step that returns early leaves no work beside the server's stream either.
+struct ServerJoin {
+    fld_server_s *s;
+    size_t nside;
+    bool done = false;
+    ~ServerJoin() {
+        if (!done) (void)server_join(s, nside);
+    }
+};
 
 // The device tables of the multi-grid launches (allocated on first use).
 fld_status server_multi_tables(fld_server_s *s) {
@@ -2387,6 +2399,7 @@ fld_status fld_server_add(fld_server s, fld_grid g, long long tag) {
     e.warm = warmup_of(g, p);
     e.am = p->anderson;
     if (e.am > 0 && (st = ensure_anderson(g, e.am)) != FLD_OK) return st;
+    if ((st = server_dots(s, (int)s->active.size() + 1)) != FLD_OK) return st;
     if ((st = preallocate(g, p)) != FLD_OK) return st;
     e.ctl.precision = p->precision;
     if (p->anderson <= 1) e.ctl.scale_windows(std::max(g->nx, std::max(g->ny, g->nz)), e.ce);
@@ -2455,6 +2468,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
         // -- one block of iterations per active grid, grids spread over the pool
         FLD_CK(cudaEventRecord(s->fork, s->bs));
         const size_t nside = s->side.size() < n ? s->side.size() : n;
+        ServerJoin joined{s, nside};
         for (size_t i = 0; i < nside; ++i) FLD_CK(cudaStreamWaitEvent(s->side[i], s->fork, 0));
         std::vector<int> k(n);
         std::vector<char> mixing(n, 0);
@@ -2704,7 +2718,6 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
         // readback, then each grid's weights and mix (same kernels and order
         // as fld_solve, so a grid's iterates are those of its solo solve)
         std::vector<double> dots(n * kAndersonMax);
-        if ((st = server_dots(s, (int)n)) != FLD_OK) return st;
         bool any_mix = false;
         for (size_t i = 0; i < n; ++i) {
             if (!mix_now[i]) continue;
@@ -2751,6 +2764,7 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
             }
         }
         if (any_mix) FLD_CK(server_join(s, nside));
+        joined.done = true;
         for (size_t r = retire.size(); r-- > 0;) {
             ServerEntry &e = s->active[retire[r].first];
             if (e.fam == FAM_F64 && (st = sync_family(e.g, FAM_FF)) != FLD_OK) return st;   // as fld_solve
