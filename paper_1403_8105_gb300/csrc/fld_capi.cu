@@ -1635,8 +1635,7 @@ fld_status iterate_replayed(fld_grid_s *g, Family fam, const PassParams &pp, int
     if (capturing != cudaStreamCaptureStatusNone) return FLD_OK;
     if (!(e.fam == fam && e.iters == iters && same_params(e.p, pp))) {
         if (e.exec) {
-            FLD_CK(cudaStreamSynchronize(g->stream));   // it may still run
-            cudaGraphExecDestroy(e.exec);
+            cudaGraphExecDestroy(e.exec);   // (one that still runs is freed when it has)
             e.exec = nullptr;
         }
         e.fam = fam;
