@@ -11,6 +11,7 @@
 #include <string.h>
 
 #include <dlfcn.h>
+#include <limits.h>
 #include <stdlib.h>
 
 #include <algorithm>
@@ -104,7 +105,7 @@ struct fld_grid_s {
     bool lo_live = false;                        // phlo may be non-zero
     GraphEntry graphs[4];
     GraphEntry replay;                           // fld_iterate on small grids (iterate_replayed)
-    int replay_calls = 0;                        // calls in a row with its family, count and parameters
+    int replay_calls = 0;                        // calls in a row with its family, count and parameters; < 0: no graph to be had
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, evb0 = nullptr, evb1 = nullptr;
     long long kernels = 0;                       // kernel launches issued so far
     fld_grid_s *coarse = nullptr;                // nested solves: the next 2x coarser grid (owned)
@@ -1644,23 +1645,29 @@ fld_status iterate_replayed(fld_grid_s *g, Family fam, const PassParams &pp, int
         g->replay_calls = 0;
     }
     if (g->replay_calls < kReplayAfter) {
-        ++g->replay_calls;
+        if (g->replay_calls >= 0) ++g->replay_calls;
         return FLD_OK;
     }
     if (!e.exec) {
         CaptureStream cap;
-        FLD_CK(cudaStreamCreateWithFlags(&cap.s, cudaStreamNonBlocking));
-        const OnStream on(g, cap.s);
         cudaGraph_t graph = nullptr;
-        FLD_CK(cudaStreamBeginCapture(cap.s, cudaStreamCaptureModeThreadLocal));
-        const fld_status st = enqueue_iterations(g, fam, pp, iters);
-        cudaError_t ce = cudaStreamEndCapture(cap.s, &graph);
+        fld_status st = FLD_OK;
+        cudaError_t ce = cudaStreamCreateWithFlags(&cap.s, cudaStreamNonBlocking);
+        if (ce == cudaSuccess) ce = cudaStreamBeginCapture(cap.s, cudaStreamCaptureModeThreadLocal);
+        if (ce == cudaSuccess) {
+            const OnStream on(g, cap.s);
+            st = enqueue_iterations(g, fam, pp, iters);
+            ce = cudaStreamEndCapture(cap.s, &graph);
+        }
         if (st == FLD_OK && ce == cudaSuccess) ce = cudaGraphInstantiate(&e.exec, graph, 0);
         if (graph) cudaGraphDestroy(graph);
-        if (st != FLD_OK) return st;
-        if (ce != cudaSuccess) {
+        if (st != FLD_OK || ce != cudaSuccess) {
+            // no room for a graph: the launches need none, for this count and these
+            // parameters from now on
+            (void)cudaGetLastError();
             e.exec = nullptr;
-            return cuda_fail(ce, "the graph of the iterations");
+            g->replay_calls = INT_MIN;
+            return FLD_OK;
         }
     }
     FLD_CK(cudaGraphLaunch(e.exec, g->stream));
