@@ -824,6 +824,10 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
             if (rep > 0) t = std::min(t, 1e3 * ms / n);
         }
         if (exec) cudaGraphExecDestroy(exec);
+        if (ce == cudaErrorMemoryAllocation) {   // no room for this one's graph: not among the choices
+            (void)cudaGetLastError();
+            continue;
+        }
         if (ce != cudaSuccess) return cuda_fail(ce, "timing a sweep");
         if (cand == -1 && early) c.us_launched = t;
         if (t < best) {
@@ -831,6 +835,10 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
             c.tiled = cand;
             c.early = early;
         }
+    }
+    if (isinf(best)) {   // none could be timed: the defaults, to be tuned another time
+        *out = TuneChoice{};
+        return FLD_OK;
     }
     if (ncfg > 0) g->tiled_used = true;   // surface a timeout of the timed blocked launches at the next check
     c.us_best = best;
@@ -896,7 +904,7 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
             std::lock_guard<std::mutex> lk(g_tune_mu);
             auto it = g_tune.find(key);   // another thread may have tuned it meanwhile: keep the first
             if (it != g_tune.end()) c = it->second;
-            else tune_store_locked(key, c);
+            else if (c.us_best > 0.0) tune_store_locked(key, c);
         }
         if (p->temporal_depth == 0) {
             if ((st = ensure_tiled(g, c.tiled)) != FLD_OK) return st;

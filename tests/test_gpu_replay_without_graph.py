@@ -1,6 +1,7 @@
 """fld_iterate where no graph can be made (its instantiation fails for want of
-memory): the call goes on with launches, with the same bits.  The failure is a
-fake of cudaGraphInstantiate, preloaded into a process of its own."""
+memory): the call goes on with launches, with the same bits, whether the graph
+is that of a replay or those a new shape's forms are timed by.  The failure is
+a fake of cudaGraphInstantiate, preloaded into a process of its own."""
 import os
 import subprocess
 import sys
@@ -34,6 +35,22 @@ import ctypes, sys, numpy as np
 sys.path[:0] = [{root!r}, {tests!r}]
 import test_gpu_replay as t
 fake = ctypes.CDLL({fake!r})
+# a shape that was never tuned, and cannot be: no candidate's graph can be made
+import os
+os.environ["FLD_TUNE_CACHE"] = {cache!r}
+fake.fake_refuse(1)
+first = []
+with t.grid(None) as g:
+    g.iterate(t.par(1.4, "pair"), 8)
+    first.append(g.get_state())
+fake.fake_refuse(0)
+assert not os.path.exists({cache!r})
+with t.grid(None) as g:
+    g.iterate(t.par(1.4, "pair"), 8)          # tuned now
+    first.append(g.get_state())
+assert os.path.exists({cache!r})
+assert np.array_equal(first[0][0], first[1][0]) and np.array_equal(first[0][1], first[1][1])
+start = fake.fake_refusals()
 with t.grid(None) as g, t.grid(None) as ref:
     for x in (g, ref):
         for n in (8, 3, 2):
@@ -45,7 +62,7 @@ with t.grid(None) as g, t.grid(None) as ref:
             ref.iterate(t.par(1.4), n)
         a, b = g.get_state(), ref.get_state()
         assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1]), k
-    assert fake.fake_refusals() == 1          # asked for once, not on every call
+    assert fake.fake_refusals() == start + 1          # asked for once, not on every call
     fake.fake_refuse(0)
     for k in range(4):                        # another count: graphs again
         g.iterate(t.par(1.4), 5)
@@ -62,7 +79,7 @@ def test_launches_go_on_where_no_graph_can_be_made(tmp_path):
     src.write_text(_FAKE)
     subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-o", str(so), str(src), "-ldl"], check=True)
     tests = os.path.dirname(os.path.abspath(__file__))
-    code = _CHILD.format(root=os.path.dirname(tests), tests=tests, fake=str(so))
+    code = _CHILD.format(root=os.path.dirname(tests), tests=tests, fake=str(so), cache=str(tmp_path / "tune.txt"))
     r = subprocess.run([sys.executable, "-c", code], timeout=600, capture_output=True, text=True,
                        env=dict(os.environ, LD_PRELOAD=str(so)))
     assert r.returncode == 0, r.stderr[-2000:]
