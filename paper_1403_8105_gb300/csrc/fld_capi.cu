@@ -2104,8 +2104,17 @@ namespace {
 // Multi-grid tables a server step can fill (groups of grids with equal block
 // lengths; a further group runs grid by grid).
 constexpr int kFuseSlots = 8;
-// Voxels of active grids above which they fill the GPU together.
-constexpr long long kCrowdVoxels = 250000;
+// What the tuner chose for a grid alone, it chose for an idle GPU.  Other grids of a
+// step are in the way of two kinds of form, and the pair passes run instead: whole
+// iterations per launch, whose few hundred large CTAs fill the GPU once whatever the
+// grid's size, from the fourth grid on; and the one-unknown and late passes, which
+// spend lanes and instructions to shorten a pass, above so many voxels of all grids
+// per SM.  1536 iterations of each grid, ms, tuned / pairs.  Hi/lo: 2 grids of 32^3 8.7 / 9.7,
+// 3 11.3 / 12.0, 4 14.6 / 14.2, 8 of 20^3 25.8 / 21.7, 16 of 32^3 54 / 37.6.  FP32: 3 of 50^3
+// (2467 voxels per SM) 15.0 / 17.2, 6 of 50^3 (4934) 25.2 / 26.2, 3 of 64^3 (5174) 15.9 / 15.8,
+// 8 of 48^3 (5820) 31.9 / 31.0, 4 of 64^3 (6899) 20.6 / 17.8.
+constexpr size_t kRowsGrids = 3;
+constexpr long long kCrowd = 5200;
 
 // The state the Anderson kernels read and write for family fam.
 void anderson_state(fld_grid_s *g, Family fam, float **hi, float **lo, double **p64) {
@@ -2486,11 +2495,9 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
         for (size_t i = 0; i < nside; ++i) FLD_CK(cudaStreamWaitEvent(s->side[i], s->fork, 0));
         std::vector<int> k(n);
         std::vector<char> mixing(n, 0);
-        // the forms for small grids spend instructions and lanes to shorten a pass:
-        // with enough other grids to fill the GPU the pair passes get more done
         long long voxels = 0;
         for (const ServerEntry &e : s->active) voxels += nvox(e.g);
-        const bool crowded = voxels > kCrowdVoxels;
+        const bool crowded = n > 1 && voxels > kCrowd * s->active[0].g->nsm;
         for (size_t i = 0; i < n; ++i) {
             const ServerEntry &e = s->active[i];
             k[i] = block_len(e.res.iterations, check_len(e.fam, p->precision, e.ce), p->max_iters, e.warm);
@@ -2572,10 +2579,8 @@ fld_status fld_server_step(fld_server s, long long *tags, fld_solve_result *resu
             }
             if (slot_of[i] < 0) {
                 PassParams q = block_params(e.pp, e.res.iterations, e.warm);
+                if (n > kRowsGrids) q.rows_f32 = q.rows_fh = 0;
                 if (crowded) {
-                    // (the pair passes, launched early throughout: 16 clouds of
-                    // 32^3 to 64^3 104 -> 93 ms; whole iterations 129)
-                    q.rows_f32 = q.rows_fh = 0;
                     q.single_f32 = q.single_fh = 0;
                     q.run_f32 = q.run_fh = -1;
                     q.direct = 1;
