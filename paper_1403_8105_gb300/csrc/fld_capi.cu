@@ -772,13 +772,18 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
     const int n = 16;   // iterations per timing, a multiple of every depth
     TuneChoice c;
     double best = INFINITY;
-    // (launches that are not early lose on all but small grids: not tried there)
+    // launches that are not early lose on all but small grids; there the fastest of
+    // the launched passes is timed so too
     const bool late = nvox(g) <= kLateMaxVoxels;
-    for (int ci = -10; ci < ncfg; ++ci) {
-        const int cand = ci < -5 ? ci + 5 : ci, early = ci < -5 ? 0 : 1;
-        if ((!early || cand == -5) && !late) continue;
-        if (cand == -4 && (!rows || !early)) continue;
-        if (cand == -5 && fam == FAM_FF) continue;     // (its -2)
+    int launched = 0;                      // the fastest launched pass
+    double launched_us = INFINITY;
+    for (int ci = -5; ci <= ncfg; ++ci) {
+        const int cand = ci < ncfg ? ci : launched, early = ci < ncfg ? 1 : 0;
+        if ((cand == -5 && !late) || (cand == -4 && !rows)) continue;
+        // (the float-float passes have their one unknown per thread as -2, and only
+        // Levermore-Pomraning in two rounds has a form with five CTAs per SM)
+        if (fam == FAM_FF && (cand == -5 || (cand == -3 && (pp.lim != LIM_LP || pp.local_iters != 2)))) continue;
+        if (!early && (!late || launched == 0)) continue;
         double t = INFINITY;
         PassParams pc = pp;
         pc.quad_f32 = pc.quad_fh = cand == -2 ? 1 : 0;
@@ -830,6 +835,10 @@ fld_status tune_family(fld_grid_s *g, const fld_solve_params *p, const PassParam
         }
         if (ce != cudaSuccess) return cuda_fail(ce, "timing a sweep");
         if (cand == -1 && early) c.us_launched = t;
+        if (cand < 0 && cand != -4 && t < launched_us) {
+            launched = cand;
+            launched_us = t;
+        }
         if (t < best) {
             best = t;
             c.tiled = cand;
@@ -884,7 +893,8 @@ fld_status choose_sweeps(fld_grid_s *g, const fld_solve_params *p, PassParams *p
     }
     if (p->temporal_depth != 0 && p->check_every > 0) return FLD_OK;
     const Family fams[3] = {p->precision == FLD_PREC_PAIR ? FAM_FH : FAM_F32, FAM_FH, FAM_FF};
-    const int nfam = p->precision != FLD_PREC_MIXED ? 1 : p->temporal_depth == 0 ? 3 : 2;
+    // (on larger grids the float-float passes have one best form: launch_pass's rule)
+    const int nfam = p->precision != FLD_PREC_MIXED ? 1 : p->temporal_depth == 0 && nvox(g) <= kLateMaxVoxels ? 3 : 2;
     for (int k = 0; k < nfam; ++k) {
         const Family fam = fams[k];
         const std::string key = tune_key(g, fam, *pp);
