@@ -286,8 +286,9 @@ void fld_default_params(fld_solve_params *p);
 /* Create a grid of nx*ny*nz unknowns (each >= 1) of edge h > 0 on the
  * current CUDA device.  stream: cudaStream_t or NULL.  *out receives the
  * handle.  Allocates the solver fields on the device (about 40 bytes per
- * voxel; the FP64 fields are added on first FP64 use and the solve's
- * snapshot of its best state on the first fld_solve). */
+ * voxel, 48 on grids of up to 100,000 voxels; the FP64 fields are added on
+ * first FP64 use and the solve's snapshot of its best state on the first
+ * fld_solve). */
 fld_status fld_create_grid(int nx, int ny, int nz, double h, void *stream, fld_grid *out);
 
 /* Medium: extinction sigma_t >= 0 and albedo in [0, 1] (unpadded, float).

@@ -140,9 +140,9 @@ __device__ __forceinline__ void cell_fh(float p0, float p0lo, const float ps[6],
     D_new = Dp;
 }
 
-// Terms of the residual-form update that do not depend on D_p, shared by the
-// sweep and the residual kernel so both evaluate the same discrete equation
-// bit for bit:  A = sum_s d_s,  B = sum_s D_s d_s,  C = sum_s D_s,
+// Terms of the residual-form update that do not depend on D_p, for one unknown;
+// ff_terms_pair below forms them for two, with the same bits, in the sweeps and in the
+// residual kernel, so both evaluate the same discrete equation:  A = sum_s d_s,  B = sum_s D_s d_s,  C = sum_s D_s,
 // base = jh2 - ah2 phi_p + B/2, and the central differences.  A and B are
 // compensated sums (Ogita-Rump-Oishi style): each difference d_s =
 // phi_s - phi_p is formed exactly as a pair (TwoSum of the high words plus

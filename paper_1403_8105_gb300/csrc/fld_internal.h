@@ -190,8 +190,8 @@ static_assert(sizeof(BatchDesc) % 16 == 0, "BatchDesc is read with 16-byte loads
 
 // One grid of a multi-grid colour pass (launch_pass_multi): its layout,
 // fields and pass parameters, and where its work items start.  An item is
-// the 32 x 8 pairs of unknowns a CTA of the solo pair pass covers (one
-// z-plane); the grid's items are numbered x fastest, then y, then z.
+// 32 x 8 pairs of unknowns of one z-plane; the grid's items are numbered x
+// fastest, then y, then z.
 struct alignas(16) SweepDesc {
     Layout L;
     float *sp, *ah2, *jh2, *phi, *phlo, *D;

@@ -670,8 +670,8 @@ __global__ void __launch_bounds__(128) k_pass4(Layout L, const float *__restrict
 // table of SweepDescs.  The CTAs are persistent (all resident) and walk the
 // work items of all grids with a grid-wide stride; item i belongs to the last
 // grid whose first item is <= i (binary search over the firsts, staged in
-// shared memory).  An item is what a CTA of the solo pair pass covers and its
-// unknowns go through tile_f32 / tile_fh with the grid's own parameters, so
+// shared memory).  An item is 32 x 8 pairs of unknowns of a z-plane, which
+// go through tile_f32 / tile_fh with the grid's own parameters, so
 // every grid gets the bits of its solo passes.  The table and both counts
 // are read on the device: one captured graph of these launches serves any
 // set of grids.
@@ -952,7 +952,7 @@ __global__ void __launch_bounds__(kPassDThreads) k_pass_d(Layout L, PassIndex ix
 // the caches), in strides of all CTAs.  One voxel per thread, the sums cost as
 // much as the residual itself and left one pair of partial sums per 256 voxels
 // for the last block to add: at 256^3 fresh D, residual and final sum took 104,
-// 362 and 79 us; now 108, 168 and 7 (the residual: 422 instructions a pair, issue 54 %
+// 362 and 79 us; now 108, 179 and 7 (the residual: 448 instructions a pair, issue 49 %
 // active, 72 registers; fresh D: 370 a pair, issue 73 %).
 constexpr int kCheckThreads = 128;
 constexpr int kCheckCtas = 2128;       // two waves of the residual's seven per SM of 152
@@ -1019,8 +1019,8 @@ __global__ void k_fresh_D_d(Layout L, const double *__restrict__ sp, const doubl
 // The two running sums of a residual check (in x and y) in three words each: every
 // TwoSum's error is added to the next word, so that hundreds of terms a thread
 // leave no more than one does. (By float-float additions 980 equal terms, whose
-// roundings do not cancel, were 7e-13 off.) Packed, the two cost what two
-// float-float additions did.
+// roundings do not cancel, were 7e-13 off.) Packed, both take 11 us of the 179 at
+// 256^3 more than float-float additions (scalar: 22).
 struct Sums {
     float2 hi, lo, err;
 };
@@ -1308,10 +1308,10 @@ __global__ void k_bake_scan_negz(Layout L, const float *__restrict__ st, const f
 // predecessor divided by h three times, floored by conversions and formed 64-bit
 // indices for every sample, and marched for voxels that scatter nothing, whose
 // source is zero whatever the transmittance (62 % of the box of a sphere cloud).
-// A point light over a 160^3 cloud: 4.27 -> 0.87 ms, and 0.78 with the fraction
+// A point light over a 160^3 cloud: 4.27 -> 0.87 ms, and 0.77 with the fraction
 // saturated instead of the coordinate clamped, the sample's number counted in
 // float and 32-bit byte offsets (the same bits); an oblique light, 200^3: 8.4 ->
-// 1.9 -> 1.7 ms.  Error against 64 bits 9.8e-7 -> 6.0e-7.
+// 1.9 -> 1.7 ms.  Error against 64 bits 9.8e-7 -> 5.2e-7.
 //
 // t = (u - 1/2) + M, M = 1.5 2^23, rounds u - 1/2 to an integer in t's low bits:
 // the lower corner b (u itself if it is one: the blend is the same from either
